@@ -350,6 +350,15 @@ __device__ __forceinline__ void block_reduce(const float (&v)[K], double* sm) {
 // ---------------------------------------------------------------------------
 // Teams
 // ---------------------------------------------------------------------------
+// The warps of a team as a product sees them: warp w of n takes items w, w + n, …
+template <bool CTA>
+struct Warps {
+  static constexpr bool kCtaScope = CTA;  // every warp of the product is in one CTA
+  int w, n;
+  __device__ int warp() const { return w; }
+  __device__ int nwarps() const { return n; }
+};
+
 struct GridTeam {
   static constexpr bool kCtaScope = false;  // products span CTAs
   Barrier* bar;
@@ -365,6 +374,16 @@ struct GridTeam {
   __device__ int nwarps() const { return gridDim.x * (blockDim.x >> 5); }
   __device__ int warp() const { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
   __device__ bool leader() const { return blockIdx.x == 0 && threadIdx.x == 0; }
+  // Spread numbering: consecutive warps on consecutive CTAs.  With the plain
+  // numbering a stage with fewer items than warps fills the first SMs with 16
+  // warps each and leaves the others idle; an FP64 warp instruction takes 17
+  // cycles of its SM, so those SMs' FP64 pipes set the stage's time (Lasso,
+  // 20000 × 200, Ā product: 1300 slices on 81 of 152 SMs).  Used wherever the
+  // numbering does not decide which terms share a partial sum.
+  __device__ Warps<false> spread() const {
+    return {(int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x), nwarps()};
+  }
+  __device__ int etid() const { return spread().w * 32 + (int)(threadIdx.x & 31); }
 
   // Grid barrier with a bounded wait.  The arrival counter only grows
   // during a launch (the host zeroes it before every launch), so barrier
@@ -521,6 +540,10 @@ struct ClusterTeam {
   __device__ int nwarps() const { return (int)csize * (blockDim.x >> 5); }
   __device__ int warp() const { return (int)rank * (blockDim.x >> 5) + (threadIdx.x >> 5); }
   __device__ bool leader() const { return rank == 0 && threadIdx.x == 0; }
+  __device__ Warps<false> spread() const {  // as GridTeam::spread
+    return {(int)((threadIdx.x >> 5) * csize + rank), nwarps()};
+  }
+  __device__ int etid() const { return spread().w * 32 + (int)(threadIdx.x & 31); }
 
   __device__ bool sync() {
     __syncthreads();
@@ -608,6 +631,8 @@ struct BlockTeam {
   __device__ int nwarps() const { return blockDim.x >> 5; }
   __device__ int warp() const { return threadIdx.x >> 5; }
   __device__ bool leader() const { return threadIdx.x == 0; }
+  __device__ Warps<true> spread() const { return {warp(), nwarps()}; }
+  __device__ int etid() const { return threadIdx.x; }
   __device__ bool sync() {
     __syncthreads();
     return true;
@@ -893,7 +918,7 @@ __device__ __forceinline__ void jacobi_rows(const Team& tm, const Dev<T>& d, dou
   const int n = d.n;
   const uint8_t* __restrict__ rtype = d.rtype;
   spmv<1, false, double, T>(
-      tm, d.kn, d.kn_ci, d.kn_v,
+      tm.spread(), d.kn, d.kn_ci, d.kn_v,
       [&](int c, T v, double* acc) {
         if (c >= n) {
           double vv = (double)v;
@@ -915,15 +940,17 @@ __device__ __forceinline__ void jacobi_rows(const Team& tm, const Dev<T>& d, dou
 template <class Team, typename T>
 __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double rho_bar,
                             bool reset_iterates) {
-  const int n = d.n, m = d.m, tid = tm.tid(), nth = tm.nthreads();
+  // sums run over tid, everything else over the spread numbering
+  const int n = d.n, m = d.m, tid = tm.tid(), et = tm.etid(), nth = tm.nthreads();
+  const auto rows = tm.spread();
   double c = 1.0;
-  for (int j = tid; j < n; j += nth) {
+  for (int j = et; j < n; j += nth) {
     d.D[j] = 1.0;
     d.nrm_n[j] = 0.0;
     d.pdiag[j] = 0.0;
     d.dg[j] = 0.0;
   }
-  for (int i = tid; i < m; i += nth) {
+  for (int i = et; i < m; i += nth) {
     d.E[i] = 1.0;
     d.nrm_m[i] = 0.0;
     const double lr = d.l_raw[i], ur = d.u_raw[i];
@@ -937,26 +964,26 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     // Kn, and for the last m through the rows of Ā.
     const double cc = c;
     spmv<2, true, double, double>(
-        tm, d.kn, d.kn_ci, d.kn_raw,
+        rows, d.kn, d.kn_ci, d.kn_raw,
         [&](int col, double v, double* acc) {
           if (col < n) acc[0] = fmax(acc[0], fabs(v) * d.D[col]);
           else acc[1] = fmax(acc[1], fabs(v) * d.E[col - n]);
         },
         [&](int j, double* acc) { d.nrm_n[j] = d.D[j] * fmax(cc * acc[0], acc[1]); });
     spmv<1, true, double, double>(
-        tm, d.as, d.a_ci, d.a_raw,
+        rows, d.as, d.a_ci, d.a_raw,
         [&](int col, double v, double* acc) { acc[0] = fmax(acc[0], fabs(v) * d.D[col]); },
         [&](int i, double* acc) { d.nrm_m[i] = d.E[i] * acc[0]; });
     if (!tm.sync()) return false;
     // δ, S ← diag(δ)S, and ‖1 − δ‖∞
     double dev[1] = {0.0};
-    for (int j = tid; j < n; j += nth) {
+    for (int j = et; j < n; j += nth) {
       double dl = ruiz_delta(d.nrm_n[j]);
       d.nrm_n[j] = 0.0;
       d.D[j] *= dl;
       dev[0] = fmax(dev[0], fabs(1.0 - dl));
     }
-    for (int i = tid; i < m; i += nth) {
+    for (int i = et; i < m; i += nth) {
       double dl = ruiz_delta(d.nrm_m[i]);
       d.nrm_m[i] = 0.0;
       d.E[i] *= dl;
@@ -967,13 +994,13 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     ++passes;
     // Cost scaling γ = 1/max{mean_j ‖P̄_:,j‖∞, ‖q̄‖∞} with the new D.
     spmv<1, true, double, double>(
-        tm, d.kn, d.kn_ci, d.kn_raw,
+        rows, d.kn, d.kn_ci, d.kn_raw,
         [&](int col, double v, double* acc) {
           if (col < n) acc[0] = fmax(acc[0], fabs(v) * d.D[col]);
         },
         [&](int j, double* acc) { d.nrm_n[j] = cc * d.D[j] * acc[0]; });
     double qn[1] = {0.0};
-    for (int j = tid; j < n; j += nth) qn[0] = fmax(qn[0], fabs(cc * d.D[j] * d.q_raw[j]));
+    for (int j = et; j < n; j += nth) qn[0] = fmax(qn[0], fabs(cc * d.D[j] * d.q_raw[j]));
     if (!tm.template publish_sync<1, 1u>(qn)) return false;
     tm.template collect<1, 1u>(qn);
     double sum[1] = {0.0};
@@ -995,7 +1022,7 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     if (dev[0] <= P.eps_equil) break;
   }
   // Scaled data: P̄ = cDPD, Ā = EAD (in both Kn and Ā), q̄ = cDq, [El, Eu].
-  foreach_entry(tm, d.kn, d.kn_ci, [&](int j, int k) {
+  foreach_entry(rows, d.kn, d.kn_ci, [&](int j, int k) {
     const int col = d.kn_ci[k];
     const double v = d.kn_raw[k];
     double s;
@@ -1007,13 +1034,13 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     }
     d.kn_v[k] = T(s);
   });
-  foreach_entry(tm, d.as, d.a_ci,
+  foreach_entry(rows, d.as, d.a_ci,
                         [&](int i, int k) { d.a_v[k] = T(d.E[i] * d.a_raw[k] * d.D[d.a_ci[k]]); });
-  for (int j = tid; j < n; j += nth) {
+  for (int j = et; j < n; j += nth) {
     d.q[j] = c * d.D[j] * d.q_raw[j];
     d.Dinv[j] = 1.0 / d.D[j];
   }
-  for (int i = tid; i < m; i += nth) {
+  for (int i = et; i < m; i += nth) {
     d.Einv[i] = 1.0 / d.E[i];
     const uint8_t t = d.rtype[i];
     d.l[i] = (t & kLInf) ? -INFINITY : d.E[i] * d.l_raw[i];
@@ -1031,12 +1058,12 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     d.sc->rd_last = reset_iterates ? 0.0 : -1.0;
   }
   if (reset_iterates) {
-    for (int j = tid; j < n; j += nth) {
+    for (int j = et; j < n; j += nth) {
       d.x[j] = 0.0;
       d.dx[j] = 0.0;
       d.xt[j] = 0.0;
     }
-    for (int i = tid; i < m; i += nth) {
+    for (int i = et; i < m; i += nth) {
       d.z[i] = 0.0;
       d.y[i] = 0.0;
       d.dy[i] = 0.0;
@@ -1057,10 +1084,10 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
 // ---------------------------------------------------------------------------
 template <class Team, typename T>
 __device__ bool refresh_stage(Team& tm, const Dev<T>& d, const Params& P, double rho_bar) {
-  const int n = d.n, m = d.m, tid = tm.tid(), nth = tm.nthreads();
+  const int n = d.n, m = d.m, et = tm.etid(), nth = tm.nthreads();
   const double c = d.sc->c;
-  for (int j = tid; j < n; j += nth) d.q[j] = c * d.D[j] * d.q_raw[j];
-  for (int i = tid; i < m; i += nth) {
+  for (int j = et; j < n; j += nth) d.q[j] = c * d.D[j] * d.q_raw[j];
+  for (int i = et; i < m; i += nth) {
     const double lr = d.l_raw[i], ur = d.u_raw[i];
     const uint8_t t = (uint8_t)((lr <= -kInfBound ? kLInf : 0) | (ur >= kInfBound ? kUInf : 0) |
                                 (lr == ur ? kEq : 0));
@@ -1391,12 +1418,36 @@ __device__ void stage_out(const Dev<T>& d, const Dev<T>& sd) {
   __syncthreads();
 }
 
+// Numbering of the products that also add up the inner product (w, u) per
+// thread (the terms of one CTA share a partial sum).  The spread numbering
+// where Kn has no more chunks and no more slices than half the warps: there
+// the plain one would leave more than half of the SMs without work, and every
+// thread adds at most two terms.  Above that the sums stay grouped as the
+// rows are dealt.
+template <class Team>
+__device__ __forceinline__ Warps<Team::kCtaScope> inner_rows(const Team& tm, const Sched& S) {
+  const int half = tm.nwarps() / 2;
+  if (S.nslices <= half && S.nchunks <= half) return tm.spread();
+  return {tm.warp(), tm.nwarps()};
+}
+
 // ---------------------------------------------------------------------------
 // Stage 2: Algorithm 1 with the indirect linear solve of §3.1.
 // ---------------------------------------------------------------------------
 template <class Team, typename T>
 __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
-  const int n = d.n, m = d.m, tid = tm.tid(), nth = tm.nthreads();
+  // stages that add up terms per thread run over tid, the others over the
+  // spread numbering
+  const int n = d.n, m = d.m, tid = tm.tid(), et = tm.etid(), nth = tm.nthreads();
+  const auto rows = tm.spread();
+  // the PCG loop's own stages: an FP32 product is not bound by the arithmetic
+  // pipe, and few SMs share the gathered lines of u better than many (Lasso
+  // FP32-mixed: 42.8 ms plain, 44.5 ms spread)
+  constexpr bool kWide = sizeof(T) == sizeof(double);
+  const Warps<Team::kCtaScope> plain{tm.warp(), tm.nwarps()};
+  const auto prows = kWide ? rows : plain;
+  const int pt = kWide ? et : tid;
+  const auto krows = kWide ? inner_rows(tm, d.kn) : plain;
   const double sigma = P.sigma, alpha = P.alpha;
   const T sigT = T(sigma);
   const double c = d.sc->c;
@@ -1466,18 +1517,18 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   int cur = 0;
 
   // Right-hand-side inputs of the first iteration from the current iterates.
-  for (int i = tid; i < m; i += nth) {
+  for (int i = et; i < m; i += nth) {
     const double rh = rho[i];
     wm[i] = rh * z[i] - y[i];
     um[i] = rh * (z[i] - zt[i]) - y[i];
     dzt[i] = T(0);
   }
-  for (int j = tid; j < n; j += nth) dxt[j] = T(0);
+  for (int j = et; j < n; j += nth) dxt[j] = T(0);
   if (!tm.sync()) return false;
   if (stale) {
     // ‖Āx̄ − z̄‖∞ and ‖P̄x̄ + q̄ + Āᵀȳ‖∞ on the current iterates (§5.1, scaled)
     spmv<2, false, double, T>(
-        tm, d.kn, kn_ci, kn_v,
+        rows, d.kn, kn_ci, kn_v,
         [&](int col, T v, double* acc) {
           const double vv = (double)v;
           if (col < n) acc[0] += vv * x[col];
@@ -1488,12 +1539,12 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           d.aty[j] = acc[1];
         });
     spmv<1, false, double, T>(
-        tm, d.as, a_ci, a_v, [&](int col, T v, double* acc) { acc[0] += (double)v * x[col]; },
+        rows, d.as, a_ci, a_v, [&](int col, T v, double* acc) { acc[0] += (double)v * x[col]; },
         [&](int i, double* acc) { d.ax[i] = acc[0]; });
     if (!tm.sync()) return false;
     double res[2] = {0.0, 0.0};
-    for (int i = tid; i < m; i += nth) res[0] = fmax(res[0], fabs(d.ax[i] - z[i]));
-    for (int j = tid; j < n; j += nth) res[1] = fmax(res[1], fabs(d.px[j] + d.q[j] + d.aty[j]));
+    for (int i = et; i < m; i += nth) res[0] = fmax(res[0], fabs(d.ax[i] - z[i]));
+    for (int j = et; j < n; j += nth) res[1] = fmax(res[1], fabs(d.px[j] + d.q[j] + d.aty[j]));
     if (!tm.template publish_sync<2, 3u>(res)) return false;
     tm.template collect<2, 3u>(res);
     rp_bar = res[0];
@@ -1510,7 +1561,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     {
       T* __restrict__ r = rbuf(cur);
       spmv<2, false, double, T>(
-          tm, d.kn, kn_ci, kn_v,
+          rows, d.kn, kn_ci, kn_v,
           [&](int col, T v, double* acc) {
             const double vv = (double)v;
             if (col < n) {
@@ -1553,7 +1604,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       red3t[1] = a1;
       red3t[2] = a2;
       spmv<1, false, T, T>(
-          tm, d.as, a_ci, a_v,
+          prows, d.as, a_ci, a_v,
           [&](int col, T v, T* acc) { acc[0] += v * (r[col] * dinv[col]); },
           [&](int i, T* acc) { t[i] = rhoT[i] * acc[0]; });
     }
@@ -1585,7 +1636,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       const T* __restrict__ u = ut;
       // long rows of w stay as chunk partials: P1, the only reader, sums them
       spmv<1, false, T, T>(
-          tm, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
+          krows, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
           [&](int j, T* acc) {
             const T wj = sigT * u[j] + acc[0];
             w[j] = wj;
@@ -1651,14 +1702,14 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         // elements above go to the first threads, so on a wide team the two
         // chains run on different warps
         const bool lazy_w = d.kn.nlong > 0;
-        for (int j = tid; j < n; j += nth)
+        for (int j = pt; j < n; j += nth)
           if (!lazy_w || d.kn.lidx[j] < 0) upd(j, wc[j]);
-        for (int lr = tm.nwarps() - 1 - tm.warp(); lr < d.kn.nlong; lr += tm.nwarps()) {
+        for (int lr = prows.n - 1 - prows.w; lr < d.kn.nlong; lr += prows.n) {
           const T sum = warp_long_sum<T>(d.kn, lr, 0);
           const int j = d.kn.long_rows[lr];
           if ((threadIdx.x & 31) == 0) upd(j, sigT * u[j] + sum);
         }
-        for (int i = tid; i < m; i += nth) {
+        for (int i = pt; i < m; i += nth) {
           const T ti = rho_invT[i] * tc[i];
           const T api = first ? ti : ti + bT * ap[i];
           ap[i] = api;
@@ -1671,7 +1722,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         const T* __restrict__ u = ubuf(nxt);
         T* __restrict__ tn = ubuf(nxt) + n;
         spmv<1, false, T, T>(
-            tm, d.as, a_ci, a_v, [&](int col, T v, T* acc) { acc[0] += v * u[col]; },
+            prows, d.as, a_ci, a_v, [&](int col, T v, T* acc) { acc[0] += v * u[col]; },
             [&](int i, T* acc) { tn[i] = rhoT[i] * acc[0]; });
       }
       if (!tm.sync()) return false;
@@ -1692,7 +1743,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           g2 = fmax(g2, fabs(rj));
         }
         spmv<1, false, T, T>(
-            tm, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
+            krows, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
             [&](int j, T* acc) {
               const T wj = sigT * u[j] + acc[0];
               wn[j] = wj;
@@ -1759,7 +1810,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     }
 
     // --- U: Algorithm 1 steps 5–7, y in the form ρ(v − Π(v)) of Eq. (zy-update)
-    for (int j = tid; j < n; j += nth) {
+    for (int j = et; j < n; j += nth) {
       const double xtj = xt[j] + (double)dxt[j];
       xt[j] = xtj;
       dxt[j] = T(0);
@@ -1767,7 +1818,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       d.dx[j] = xn - x[j];
       x[j] = xn;
     }
-    for (int i = tid; i < m; i += nth) {
+    for (int i = et; i < m; i += nth) {
       const double rh = rho[i];
       const double zti = zt[i] + (double)dzt[i];
       zt[i] = zti;
@@ -1792,7 +1843,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       const double* __restrict__ dxp = d.dx;
       const double* __restrict__ dyp = d.dy;
       spmv<4, false, double, T>(
-          tm, d.kn, kn_ci, kn_v,
+          rows, d.kn, kn_ci, kn_v,
           [&](int col, T v, double* acc) {
             const double vv = (double)v;
             if (col < n) {
@@ -1814,7 +1865,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
             d.atdy[j] = acc[3];
           });
       spmv<3, false, double, T>(
-          tm, d.as, a_ci, a_v,
+          rows, d.as, a_ci, a_v,
           [&](int col, T v, double* acc) {
             const double vv = (double)v;
             acc[0] += vv * x[col];
@@ -1915,7 +1966,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       if (rn > P.rho_tol * rho_bar || rn < rho_bar / P.rho_tol) {
         rho_bar = rn;
         ++rho_updates;
-        for (int i = tid; i < m; i += nth) {
+        for (int i = et; i < m; i += nth) {
           const double rh = rho_of(d.rtype[i], rho_bar);
           d.rho[i] = rh;
           d.rho_inv[i] = 1.0 / rh;
@@ -1939,11 +1990,11 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   }
 
   // --- unscale (Eq. pb:scaled_qp) and certificates (§5.1)
-  for (int j = tid; j < n; j += nth) {
+  for (int j = et; j < n; j += nth) {
     d.x_out[j] = d.D[j] * x[j];
     d.dcert[j] = status == kDualInf ? d.D[j] * d.dx[j] : 0.0;
   }
-  for (int i = tid; i < m; i += nth) {
+  for (int i = et; i < m; i += nth) {
     const double Ei = d.E[i];
     d.z_out[i] = z[i] * d.Einv[i];
     d.y_out[i] = Ei * y[i] / c;

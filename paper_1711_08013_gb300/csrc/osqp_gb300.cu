@@ -153,11 +153,14 @@ __global__ void __launch_bounds__(kThreads)
                 unsigned long long timeout_ns) {
   __shared__ double sm[kSmemDoubles];
   GridTeam tm{bar, err, part, sm, timeout_ns, 0, 0u};
+  // the numbering of the solve's own product (see admm_stage)
+  Warps<false> numbering{tm.warp(), tm.nwarps()};
+  if constexpr (sizeof(T) == sizeof(double)) numbering = KN ? inner_rows(tm, S) : tm.spread();
   for (int r = 0; r < reps; ++r) {
     T acc1 = T(0);
     if constexpr (KN) {
       spmv<1, false, T, T>(
-          tm, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * x[col]; },
+          numbering, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * x[col]; },
           [&](int j, T* acc) {
             const T wj = x2[j] * x[j] + acc[0];
             y[j] = wj;
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(kThreads)
           NoLong{}, LazyTag{});
     } else {
       spmv<1, false, T, T>(
-          tm, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * (x[col] * x2[col]); },
+          numbering, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * (x[col] * x2[col]); },
           [&](int i, T* acc) {
             y[i] = x2[i] * acc[0];
             acc1 += y[i];
