@@ -176,15 +176,53 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
 }
 
 // Block-wide reduction of K slots; slot k is a max when bit k of MAXMASK is
-// set, else a sum.  Max slots: integer keys combined by warp shuffles.  Sum
-// slots (at most kMaxSumSlots): every thread stages its value in shared
-// memory and one warp per slot adds the column (16 values per lane, then a
+// set, else a sum.  Every thread stages its value of a slot in shared memory
+// and one warp per slot reduces the column (16 values per lane, then a
 // 5-level shuffle tree), about a quarter of the FP64 instructions of a
-// per-warp shuffle tree.  Result left in sm[32*kMaxRed + k].  All threads
-// call it.
+// per-warp shuffle tree.  Max slots reduce order-preserving integer keys; a
+// reduction of more slots than the staging area holds combines them by warp
+// shuffles first.  Result left in sm[32*kMaxRed + k].  All threads call it.
 template <int K, unsigned MAXMASK>
 __device__ __forceinline__ void block_reduce(const double (&v)[K], double* sm) {
   static_assert(K <= kMaxRed, "too many reduction slots");
+  if constexpr (K <= kMaxSumSlots) {
+    // one warp per slot, the maxima beside the sums (a max slot that every
+    // warp first combined by shuffles cost about 250 cycles before the
+    // barrier and as much again on the warp that also adds a sum)
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double* stage = sm + 34 * kMaxRed;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      stage[k * kThreads + threadIdx.x] =
+          ((MAXMASK >> k) & 1u) ? __longlong_as_double((long long)dkey(v[k])) : v[k];
+    __syncthreads();
+    if (wid < K) {
+      const double* col = stage + wid * kThreads;
+      double t[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) t[u] = col[lane + 32 * u];
+      if ((MAXMASK >> wid) & 1u) {
+        unsigned long long x = (unsigned long long)__double_as_longlong(t[0]);
+#pragma unroll
+        for (int u = 1; u < 16; ++u)
+          x = umax64(x, (unsigned long long)__double_as_longlong(t[u]));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x = umax64(x, __shfl_xor_sync(0xffffffffu, x, off));
+        if (lane == 0) sm[32 * kMaxRed + wid] = dunkey(x);
+      } else {
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+          for (int u = 0; u < w; ++u) t[u] += t[u + w];
+        double x = t[0];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if (lane == 0) sm[32 * kMaxRed + wid] = x;
+      }
+    }
+    __syncthreads();
+    return;
+  }
   constexpr int S = K - __builtin_popcount(MAXMASK & ((1u << K) - 1u));
   static_assert(S <= kMaxSumSlots, "too many sum slots");
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -359,15 +397,23 @@ struct Warps {
   __device__ int nwarps() const { return n; }
 };
 
+// A value that another CTA stored before a barrier that this thread's warp has
+// passed; ordered after the wait for the compiler too.
+__device__ __forceinline__ double ld_partial(const double* p) {
+  double v;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+
 struct GridTeam {
   static constexpr bool kCtaScope = false;  // products span CTAs
   Barrier* bar;
   int* err;
-  double* part;  // [2][gridDim.x][kMaxRed]
+  double* part;  // [2][kMaxRed][gridDim.x]: a slot's partials are contiguous
   double* sm;
   unsigned long long timeout_ns;
   int buf;
-  unsigned int target;  // barrier count × gridDim.x reached so far (thread 0)
+  unsigned int target;  // barrier count × gridDim.x reached so far (warp 0)
 
   __device__ int nthreads() const { return gridDim.x * blockDim.x; }
   __device__ int tid() const { return blockIdx.x * blockDim.x + threadIdx.x; }
@@ -394,29 +440,41 @@ struct GridTeam {
   // kBarrierPoison to the counter, which releases every waiter at once; a
   // counter at or above kBarrierPoison makes every CTA stop at its barrier.
   static constexpr unsigned int kBarrierPoison = 0x80000000u;
-  __device__ bool sync() {
-    __syncthreads();
-    int* flag = reinterpret_cast<int*>(sm + 34 * kMaxRed - 1);
-    if (threadIdx.x == 0) {
-      target += gridDim.x;
-      unsigned int c;
+  static constexpr int kCollectPer = 5;  // partials per lane loaded together (152 CTAs)
+  // Warp 0, all lanes together: arrive and wait; 0 on a timeout.  Lane 0 does
+  // the memory accesses and the others follow its value, so that the warp
+  // stays converged for the loads that come next.
+  __device__ int warp_arrive_wait() {
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    target += gridDim.x;
+    unsigned int c = 0u;
+    if (lane0)
       asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(c) : "l"(&bar->count) : "memory");
-      c += 1u;
-      if (c < target) {
-        const unsigned long long t0 = gtimer();
-        unsigned int spins = 0;
-        for (;;) {
+    c = __shfl_sync(0xffffffffu, c, 0) + 1u;
+    if (c < target) {
+      const unsigned long long t0 = gtimer();
+      unsigned int spins = 0;
+      for (;;) {
+        if (lane0) {
           asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(c) : "l"(&bar->count) : "memory");
-          if (c >= target) break;
-          if ((++spins & 255u) == 0 && gtimer() - t0 > timeout_ns) {
+          if (c < target && (++spins & 255u) == 0 && gtimer() - t0 > timeout_ns) {
             atomicExch(err, kDevBarrierTimeout);
             atomicAdd(&bar->count, kBarrierPoison);
             c = kBarrierPoison;
-            break;
           }
         }
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= target) break;
       }
-      *flag = c < kBarrierPoison ? 1 : 0;
+    }
+    return c < kBarrierPoison ? 1 : 0;
+  }
+  __device__ bool sync() {
+    __syncthreads();
+    int* flag = reinterpret_cast<int*>(sm + 34 * kMaxRed - 1);
+    if (threadIdx.x < 32) {
+      const int ok = warp_arrive_wait();
+      if (threadIdx.x == 0) *flag = ok;
     }
     __syncthreads();
     return *flag != 0;
@@ -434,8 +492,88 @@ struct GridTeam {
   __device__ void publish(const V (&v)[K]) {
     block_reduce<K, MAXMASK>(v, sm);
     if (threadIdx.x < K)
-      part[((size_t)buf * gridDim.x + blockIdx.x) * kMaxRed + threadIdx.x] =
+      part[((size_t)buf * kMaxRed + threadIdx.x) * gridDim.x + blockIdx.x] =
           sm[32 * kMaxRed + threadIdx.x];
+  }
+
+  // Reduction of at most four slots whose results only one thread turns into
+  // scalars: f(results) runs on thread 0 of every CTA, with its writes visible
+  // to the CTA on return.  Warp 0 waits for the grid, combines the partials
+  // and runs f in one go, while the other warps wait at a single CTA barrier
+  // (publish_sync, collect and a scalar step after it take four).  The
+  // order of the sums is collect's.
+  template <int K, unsigned MAXMASK, bool DBL = true, bool MIRROR = false, typename V, class F>
+  __device__ bool reduce(const V (&v)[K], F f) {
+    static_assert(K <= 4, "four slots at most");
+    publish<K, MAXMASK>(v);
+    __syncthreads();
+    int* flag = reinterpret_cast<int*>(sm + 34 * kMaxRed - 1);
+    if (threadIdx.x < 32) {
+      const int lane = threadIdx.x, nb = gridDim.x, per = (nb + 31) >> 5;
+      const int ok = warp_arrive_wait();
+      __syncwarp();  // every lane's partial loads after lane 0's acquire
+      double res[K];
+      double y[K][kCollectPer];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const double* src = part + ((size_t)buf * kMaxRed + k) * nb;
+#pragma unroll
+        for (int u = 0; u < kCollectPer; ++u) {
+          const int b = lane + 32 * u;
+          y[k][u] = b < nb ? ld_partial(src + b) : (((MAXMASK >> k) & 1u) ? -INFINITY : 0.0);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const double* src = part + ((size_t)buf * kMaxRed + k) * nb;
+        if ((MAXMASK >> k) & 1u) {
+          unsigned long long x = dkey(y[k][0]);
+#pragma unroll
+          for (int u = 1; u < kCollectPer; ++u)
+            if (u < per) x = umax64(x, dkey(y[k][u]));
+#pragma unroll 1
+          for (int b = lane + 32 * kCollectPer; b < nb; b += 32) x = umax64(x, dkey(ld_partial(src + b)));
+          y[k][0] = __longlong_as_double((long long)x);
+        } else {
+          double x = y[k][0];
+#pragma unroll
+          for (int u = 1; u < kCollectPer; ++u)
+            if (u < per) x += y[k][u];
+#pragma unroll 1
+          for (int b = lane + 32 * kCollectPer, u = kCollectPer; u < per; b += 32, ++u)
+            x += b < nb ? ld_partial(src + b) : 0.0;
+          y[k][0] = x;
+        }
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const double o = __shfl_xor_sync(0xffffffffu, y[k][0], off);
+          if ((MAXMASK >> k) & 1u)
+            y[k][0] = __longlong_as_double(
+                (long long)umax64((unsigned long long)__double_as_longlong(y[k][0]),
+                                  (unsigned long long)__double_as_longlong(o)));
+          else
+            y[k][0] += o;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        res[k] = ((MAXMASK >> k) & 1u)
+                     ? dunkey((unsigned long long)__double_as_longlong(y[k][0]))
+                     : y[k][0];
+        if (MIRROR && lane == 0)
+          mirror_store(sm, k, ((MAXMASK >> k) & 1u) ? ff{(float)res[k], 0.0f} : ff_of(res[k]));
+      }
+      if (lane == 0) {
+        *flag = ok;
+        f(res);
+      }
+    }
+    __syncthreads();
+    buf ^= 1;
+    return *flag != 0;
   }
 
   // Combine the partials of the last publish (after a sync).  Every CTA runs
@@ -449,7 +587,7 @@ struct GridTeam {
     const int nb = gridDim.x;
     for (int k = wid; k < K; k += nw) {
       const bool mx = (MAXMASK >> k) & 1u;
-      const double* src = part + (size_t)buf * nb * kMaxRed + k;
+      const double* src = part + ((size_t)buf * kMaxRed + k) * nb;
       // the ⌈nb/32⌉ partials of a lane, loaded together, then combined in
       // lane order (no FP64 work on absent partials)
       const int per = (nb + 31) >> 5;
@@ -457,7 +595,7 @@ struct GridTeam {
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
         const int b = lane + 32 * u;
-        y[u] = (u < per && b < nb) ? __ldcg(src + (size_t)b * kMaxRed) : (mx ? -INFINITY : 0.0);
+        y[u] = (u < per && b < nb) ? __ldcg(src + b) : (mx ? -INFINITY : 0.0);
       }
       if (mx) {
         unsigned long long x = dkey(y[0]);
@@ -582,6 +720,17 @@ struct ClusterTeam {
     return sync();
   }
 
+  // as GridTeam::reduce
+  template <int K, unsigned MAXMASK, bool DBL = true, bool MIRROR = false, typename V, class F>
+  __device__ bool reduce(const V (&v)[K], F f) {
+    if (!publish_sync<K, MAXMASK>(v)) return false;
+    double res[K];
+    collect<K, MAXMASK, MIRROR>(res);
+    if (threadIdx.x == 0) f(res);
+    __syncthreads();
+    return true;
+  }
+
   template <int K, unsigned MAXMASK, typename V>
   __device__ void publish(const V (&v)[K]) {
     block_reduce<K, MAXMASK>(v, sm);
@@ -651,6 +800,19 @@ struct BlockTeam {
       block_reduce<K, MAXMASK, DBL>(v, sm);
     else
       block_reduce<K, MAXMASK>(v, sm);
+    return true;
+  }
+  // as GridTeam::reduce; without an FP64 result (DBL false) there are no
+  // scalars for one warp to form and f is not run
+  template <int K, unsigned MAXMASK, bool DBL = true, bool MIRROR = false, typename V, class F>
+  __device__ bool reduce(const V (&v)[K], F f) {
+    publish_sync<K, MAXMASK, DBL>(v);
+    if constexpr (DBL) {
+      double res[K];
+      collect<K, MAXMASK, MIRROR>(res);
+      if (threadIdx.x == 0) f(res);
+      __syncthreads();
+    }
     return true;
   }
   // the FP32 copies (MIRROR) are left by the FP32 block_reduce itself
@@ -842,14 +1004,13 @@ __device__ __forceinline__ void spmv(const Team& tm, const Sched& S, const int* 
   }
 }
 
-// Sum of long row lr's partial value v after the LAZY product that stored
+// Sum of a long row's partial value v (chunks r.x … r.x + r.y − 1) after the LAZY product that stored
 // them (a team barrier in between), by one warp: lane k adds chunks k, k+32,
 // … in order, then a fixed xor-shuffle tree, so every lane holds the same
 // total.  All lanes of the warp call it.
 template <typename AT>
-__device__ __forceinline__ AT warp_long_sum(const Sched& S, int lr, int v) {
+__device__ __forceinline__ AT warp_long_sum(const Sched& S, int2 r, int v) {
   const int lane = threadIdx.x & 31;
-  const int2 r = S.lrange[lr];
   AT acc = AT(0);
   for (int k = lane; k < r.y; k += 32) acc += (AT)__ldcg(S.cpart + (size_t)(r.x + k) * kMaxNV + v);
 #pragma unroll
@@ -1448,19 +1609,24 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   const auto prows = kWide ? rows : plain;
   const int pt = kWide ? et : tid;
   const auto krows = kWide ? inner_rows(tm, d.kn) : plain;
+  // this warp's first long row of w (see P1), kept where its table entries
+  // cost an L2 trip per use and registers are left
+  constexpr bool kKeepRow = kWide && !Team::kCtaScope;
+  const int lr0 = prows.n - 1 - prows.w;
+  const int lr0_row = kKeepRow && lr0 < d.kn.nlong ? d.kn.long_rows[lr0] : 0;
+  const int2 lr0_range = kKeepRow && lr0 < d.kn.nlong ? d.kn.lrange[lr0] : make_int2(0, 0);
   const double sigma = P.sigma, alpha = P.alpha;
   const T sigT = T(sigma);
   const double c = d.sc->c;
   double rho_bar = d.sc->rho_bar;
   // FP64 mode: scalars of the PCG recurrence (γ, α, β, tolerance, and α, β
-  // and the stop flag handed to every thread), updated by warp 0 of each CTA
+  // and the stop flag handed to every thread), updated by thread 0 of each CTA
   // after each reduction: every CTA derives the same values from the same
   // reduced inputs, and the narrow FP64 pipe runs the divisions once per CTA
   // rather than once per warp.
   double* scal = tm.sm + kScalOff;
   T* scalT = reinterpret_cast<T*>(scal + 5);
   int* sflag = reinterpret_cast<int*>(scal + 7);
-  const bool warp0 = (threadIdx.x >> 5) == 0;
   // FP32-mixed mode: every thread runs the recurrence itself, in
   // double-float arithmetic on FP32 instructions, from the reduced values
   // that the reduction leaves as double-float pairs (identical inputs and
@@ -1585,7 +1751,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // w = Ku and the two inner products (r,u), (w,u).  r, s, w and t are
     // double-buffered so that gathers never see a vector being rewritten.
     // --- A0: u = M⁻¹r, t = RĀu; (r,u), ‖r‖∞, ‖b‖∞
-    double red3[3];
     T red3t[3];
     {
       const T* __restrict__ r = rbuf(cur);
@@ -1608,20 +1773,18 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           [&](int col, T v, T* acc) { acc[0] += v * (r[col] * dinv[col]); },
           [&](int i, T* acc) { t[i] = rhoT[i] * acc[0]; });
     }
-    if (!tm.template publish_sync<3, 6u>(red3t)) return false;
-    tm.template collect<3, 6u, kF32>(red3);
-    if (warp0) {
-      // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
-      const double bnorm = red3[2];
-      const double tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
-                              have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
-                                         : 0.1 * P.pcg_kappa * bnorm);
-      scal[0] = red3[0];  // γ = (r, M⁻¹r)
-      scal[3] = tol;
-      if (kF32 && threadIdx.x == 0) *ftol = (float)tol;
-      if (threadIdx.x == 0) *sflag = !(red3[1] > tol);
-    }
-    __syncthreads();
+    if (!tm.template reduce<3, 6u, true, kF32>(red3t, [&](const double (&red3)[3]) {
+          // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
+          const double bnorm = red3[2];
+          const double tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
+                                  have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
+                                             : 0.1 * P.pcg_kappa * bnorm);
+          scal[0] = red3[0];  // γ = (r, M⁻¹r)
+          scal[3] = tol;
+          if (kF32) *ftol = (float)tol;
+          *sflag = !(red3[1] > tol);
+        }))
+      return false;
     bool done = *sflag != 0;
     if constexpr (kF32) {
       cg_g = ff{fmir[0], fmir[1]};
@@ -1629,7 +1792,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     }
     if (!done) {
       // --- W: w = Ku, (w,u)
-      double red1[1] = {0.0};
       T wacc = T(0);
       T* __restrict__ w = wbuf(cur);
       const T* __restrict__ ut = ubuf(cur);
@@ -1647,8 +1809,15 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           },
           NoLong{}, LazyTag{});
       const T red1t[1] = {wacc};
-      if (!tm.template publish_sync<1, 0u, !kF32>(red1t)) return false;
-      tm.template collect<1, 0u, kF32>(red1);
+      if (!tm.template reduce<1, 0u, !kF32, kF32>(red1t, [&](const double (&red1)[1]) {
+            if (kF32) return;
+            const double a = red1[0] > 0.0 ? scal[0] / red1[0] : 0.0;
+            scal[1] = a;
+            scalT[0] = T(a);
+            scalT[1] = T(0);
+            *sflag = !(red1[0] > 0.0);
+          }))
+        return false;
       if constexpr (kF32) {
         // α = γ/(w,u), β = 0; every thread, from the pair of (w,u)
         const ff wu{fmir[0], fmir[1]};
@@ -1660,14 +1829,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           cg_ia = ff_mul(wu, cg_ig);  // 1/α
         }
       } else {
-        if (warp0) {
-          const double a = red1[0] > 0.0 ? scal[0] / red1[0] : 0.0;
-          scal[1] = a;
-          scalT[0] = T(a);
-          scalT[1] = T(0);
-          if (threadIdx.x == 0) *sflag = !(red1[0] > 0.0);
-        }
-        __syncthreads();
         done = *sflag != 0;
       }
     }
@@ -1687,15 +1848,22 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         const T* __restrict__ tc = ubuf(cur) + n;
         const T* __restrict__ u = ubuf(cur);
         T* __restrict__ un = ubuf(nxt);
-        auto upd = [&](int j, T wj) {
-          const T pj = first ? u[j] : u[j] + bT * pv[j];
-          const T sj = first ? wj : wj + bT * sc[j];
+        // the inputs of element j but w_j, fetched together
+        struct In {
+          T u, p, s, dx, r, di;
+        };
+        auto fetch = [&](int j) {
+          return In{u[j], first ? T(0) : pv[j], first ? T(0) : sc[j], dxt[j], rc[j], dinv[j]};
+        };
+        auto upd = [&](int j, T wj, const In& e) {
+          const T pj = first ? e.u : e.u + bT * e.p;
+          const T sj = first ? wj : wj + bT * e.s;
           pv[j] = pj;
           sn[j] = sj;
-          dxt[j] += aT * pj;
-          const T rj = rc[j] - aT * sj;
+          dxt[j] = e.dx + aT * pj;
+          const T rj = e.r - aT * sj;
           rn[j] = rj;
-          un[j] = rj * dinv[j];
+          un[j] = rj * e.di;
         };
         // w = Ku; its long rows are left as the product's chunk partials and
         // summed here, one warp per row, taken from the last warp down: the
@@ -1703,11 +1871,22 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         // chains run on different warps
         const bool lazy_w = d.kn.nlong > 0;
         for (int j = pt; j < n; j += nth)
-          if (!lazy_w || d.kn.lidx[j] < 0) upd(j, wc[j]);
+        {
+          // (the row kind is fetched beside the inputs, not before them)
+          const bool mine = !lazy_w || d.kn.lidx[j] < 0;
+          const T wj = wc[j];
+          const In e = fetch(j);
+          if (mine) upd(j, wj, e);
+        }
         for (int lr = prows.n - 1 - prows.w; lr < d.kn.nlong; lr += prows.n) {
-          const T sum = warp_long_sum<T>(d.kn, lr, 0);
-          const int j = d.kn.long_rows[lr];
-          if ((threadIdx.x & 31) == 0) upd(j, sigT * u[j] + sum);
+          // place of the row known in advance; its inputs travel with the
+          // chunk partials (a dependent chain of L2 trips otherwise)
+          const bool kept = kKeepRow && lr == lr0;
+          const int j = kept ? lr0_row : d.kn.long_rows[lr];
+          const int2 rg = kept ? lr0_range : d.kn.lrange[lr];
+          const In e = fetch(j);
+          const T sum = warp_long_sum<T>(d.kn, rg, 0);
+          if ((threadIdx.x & 31) == 0) upd(j, sigT * e.u + sum, e);
         }
         for (int i = pt; i < m; i += nth) {
           const T ti = rho_invT[i] * tc[i];
@@ -1729,7 +1908,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       ++j_it;
       ++pcg_total;
       // --- P2: w = Ku, (r,u), (w,u), ‖r‖∞
-      double red2[3];
       T red2t[3];
       {
         const T* __restrict__ rn = rbuf(nxt);
@@ -1757,8 +1935,32 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         red2t[1] = g1;
         red2t[2] = g2;
       }
-      if (!tm.template publish_sync<3, 4u, !kF32>(red2t)) return false;
-      tm.template collect<3, 4u, kF32>(red2);
+      if (!tm.template reduce<3, 4u, !kF32, kF32>(red2t, [&](const double (&red2)[3]) {
+            if (kF32) return;
+            // Chronopoulos–Gear update: β = γ'/γ, α = γ'/((w,u) − βγ'/α); stop
+            // at the tolerance, the iteration cap, or a breakdown (p vanished).
+            // β = γ'/γ and γ'/α are independent of each other and correctly
+            // rounded: the FP64 PCG iteration count follows the rounding of
+            // these scalars.
+            int stop = !(red2[2] > scal[3]) || j_it >= P.pcg_max_iter;
+            if (!stop) {
+              const double gamma_n = red2[0];
+              const double beta_n = gamma_n / scal[0];
+              const double denom = red2[1] - beta_n * (gamma_n / scal[1]);
+              if (!(denom > 0.0) || !(gamma_n > 0.0)) {
+                stop = 1;
+              } else {
+                const double a = gamma_n / denom;
+                scal[0] = gamma_n;
+                scal[1] = a;
+                scal[2] = beta_n;
+                scalT[0] = T(a);
+                scalT[1] = T(beta_n);
+              }
+            }
+            *sflag = stop;
+          }))
+        return false;
       cur = nxt;
       if constexpr (kF32) {
         // Chronopoulos–Gear update in every thread, in double-float (see
@@ -1781,31 +1983,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         if (stop) break;
         continue;
       }
-      if (warp0) {
-        // Chronopoulos–Gear update: β = γ'/γ, α = γ'/((w,u) − βγ'/α); stop
-        // at the tolerance, the iteration cap, or a breakdown (p vanished).
-        // β = γ'/γ and γ'/α are independent of each other and correctly
-        // rounded: the FP64 PCG iteration count follows the rounding of
-        // these scalars.
-        int stop = !(red2[2] > scal[3]) || j_it >= P.pcg_max_iter;
-        if (!stop) {
-          const double gamma_n = red2[0];
-          const double beta_n = gamma_n / scal[0];
-          const double denom = red2[1] - beta_n * (gamma_n / scal[1]);
-          if (!(denom > 0.0) || !(gamma_n > 0.0)) {
-            stop = 1;
-          } else {
-            const double a = gamma_n / denom;
-            scal[0] = gamma_n;
-            scal[1] = a;
-            scal[2] = beta_n;
-            scalT[0] = T(a);
-            scalT[1] = T(beta_n);
-          }
-        }
-        if (threadIdx.x == 0) *sflag = stop;
-      }
-      __syncthreads();
       if (*sflag) break;
     }
 
