@@ -1726,6 +1726,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // (mixed-precision iterative refinement of the linear solve).
     {
       T* __restrict__ r = rbuf(cur);
+      T* __restrict__ u0 = ubuf(cur);
       spmv<2, false, double, T>(
           rows, d.kn, kn_ci, kn_v,
           [&](int col, T v, double* acc) {
@@ -1739,7 +1740,9 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           },
           [&](int j, double* acc) {
             const double bj = sigma * x[j] - d.q[j];
-            r[j] = T(bj - sigma * xt[j] + acc[0]);
+            const T rj = T(bj - sigma * xt[j] + acc[0]);
+            r[j] = rj;
+            u0[j] = rj * dinv[j];  // here, so that A0 gathers u instead of r and M⁻¹
             bv[j] = T(bj + acc[1]);
           });
     }
@@ -1750,18 +1753,16 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // and computes t = RĀu with u formed on the fly, and one stage that forms
     // w = Ku and the two inner products (r,u), (w,u).  r, s, w and t are
     // double-buffered so that gathers never see a vector being rewritten.
-    // --- A0: u = M⁻¹r, t = RĀu; (r,u), ‖r‖∞, ‖b‖∞
+    // --- A0: t = RĀu with the u = M⁻¹r that R left; (r,u), ‖r‖∞, ‖b‖∞
     T red3t[3];
     {
       const T* __restrict__ r = rbuf(cur);
-      T* __restrict__ u = ubuf(cur);
+      const T* __restrict__ u = ubuf(cur);
       T* __restrict__ t = ubuf(cur) + n;
       T a0 = T(0), a1 = T(0), a2 = T(0);
       for (int j = tid; j < n; j += nth) {
         const T rj = r[j];
-        const T uj = rj * dinv[j];
-        u[j] = uj;
-        a0 += rj * uj;
+        a0 += rj * u[j];
         a1 = fmax(a1, fabs(rj));
         a2 = fmax(a2, fabs(bv[j]));
       }
@@ -1770,7 +1771,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       red3t[2] = a2;
       spmv<1, false, T, T>(
           prows, d.as, a_ci, a_v,
-          [&](int col, T v, T* acc) { acc[0] += v * (r[col] * dinv[col]); },
+          [&](int col, T v, T* acc) { acc[0] += v * u[col]; },
           [&](int i, T* acc) { t[i] = rhoT[i] * acc[0]; });
     }
     if (!tm.template reduce<3, 6u, true, kF32>(red3t, [&](const double (&red3)[3]) {
@@ -1987,12 +1988,15 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     }
 
     // --- U: Algorithm 1 steps 5–7, y in the form ρ(v − Π(v)) of Eq. (zy-update)
+    // (δx and δy are read by the checks only)
+    const bool check = (k % P.check_interval == 0) || (k == P.max_iter);
     for (int j = et; j < n; j += nth) {
       const double xtj = xt[j] + (double)dxt[j];
       xt[j] = xtj;
       dxt[j] = T(0);
-      const double xn = alpha * xtj + (1.0 - alpha) * x[j];
-      d.dx[j] = xn - x[j];
+      const double xo = x[j];
+      const double xn = alpha * xtj + (1.0 - alpha) * xo;
+      if (check) d.dx[j] = xn - xo;
       x[j] = xn;
     }
     for (int i = et; i < m; i += nth) {
@@ -2000,16 +2004,16 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       const double zti = zt[i] + (double)dzt[i];
       zt[i] = zti;
       dzt[i] = T(0);
-      const double v = alpha * zti + (1.0 - alpha) * z[i] + rho_inv[i] * y[i];
+      const double yo = y[i];
+      const double v = alpha * zti + (1.0 - alpha) * z[i] + rho_inv[i] * yo;
       const double zn = fmin(fmax(v, d.l[i]), d.u[i]);
       const double yn = rh * (v - zn);
-      d.dy[i] = yn - y[i];
+      if (check) d.dy[i] = yn - yo;
       z[i] = zn;
       y[i] = yn;
       wm[i] = rh * zn - yn;
       um[i] = rh * (zn - zti) - yn;
     }
-    const bool check = (k % P.check_interval == 0) || (k == P.max_iter);
     if (!tm.sync()) return false;
     if (!check) continue;
 
