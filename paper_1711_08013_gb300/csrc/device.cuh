@@ -1107,80 +1107,81 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
   double c = 1.0;
   for (int j = et; j < n; j += nth) {
     d.D[j] = 1.0;
-    d.nrm_n[j] = 0.0;
     d.pdiag[j] = 0.0;
     d.dg[j] = 0.0;
   }
   for (int i = et; i < m; i += nth) {
     d.E[i] = 1.0;
-    d.nrm_m[i] = 0.0;
     const double lr = d.l_raw[i], ur = d.u_raw[i];
     d.rtype[i] = (uint8_t)((lr <= -kInfBound ? kLInf : 0) | (ur >= kInfBound ? kUInf : 0) |
                            (lr == ur ? kEq : 0));
   }
   if (!tm.sync()) return false;
+  // Per pass: the column norms of M = [P Aᵀ; A 0] (Kn rows give the first n,
+  // Ā rows the last m), δ, S ← diag(δ)S, then the cost factor
+  // γ = 1/max{mean_j ‖P̄_:,j‖∞, ‖q̄‖∞} with the new D.  γ needs the norms of P
+  // under the new D, which are the P half of the next pass's norms: the two
+  // halves are kept apart (nrm_n: max|P|D, aty: max|Aᵀ|E), γ is formed after
+  // the next pass's products, and one more pass over Kn ends the loop.  That
+  // takes two products and three barriers a pass instead of three and four
+  // (portfolio, 10^4 assets, FP64: 376 µs before).
   int passes = 0;
-  for (int pass = 0; pass < P.scaling_iters; ++pass) {
-    // ‖M_j‖∞ for the first n columns of M = [P Aᵀ; A 0] through the rows of
-    // Kn, and for the last m through the rows of Ā.
-    const double cc = c;
+  double dev = 0.0;
+  for (int pass = 0; P.scaling_iters > 0; ++pass) {
+    const bool last = pass == P.scaling_iters || (pass > 0 && dev <= P.eps_equil);
     spmv<2, true, double, double>(
         rows, d.kn, d.kn_ci, d.kn_raw,
         [&](int col, double v, double* acc) {
           if (col < n) acc[0] = fmax(acc[0], fabs(v) * d.D[col]);
           else acc[1] = fmax(acc[1], fabs(v) * d.E[col - n]);
         },
-        [&](int j, double* acc) { d.nrm_n[j] = d.D[j] * fmax(cc * acc[0], acc[1]); });
-    spmv<1, true, double, double>(
-        rows, d.as, d.a_ci, d.a_raw,
-        [&](int col, double v, double* acc) { acc[0] = fmax(acc[0], fabs(v) * d.D[col]); },
-        [&](int i, double* acc) { d.nrm_m[i] = d.E[i] * acc[0]; });
+        [&](int j, double* acc) {
+          d.nrm_n[j] = acc[0];
+          d.aty[j] = acc[1];
+        });
+    if (!last)
+      spmv<1, true, double, double>(
+          rows, d.as, d.a_ci, d.a_raw,
+          [&](int col, double v, double* acc) { acc[0] = fmax(acc[0], fabs(v) * d.D[col]); },
+          [&](int i, double* acc) { d.nrm_m[i] = d.E[i] * acc[0]; });
     if (!tm.sync()) return false;
+    if (pass > 0) {
+      double red[2] = {0.0, 0.0};  // Σ_j ‖P̄_:,j‖∞, ‖q̄‖∞
+      for (int j = tid; j < n; j += nth) {
+        const double cd = c * d.D[j];
+        red[0] += __dmul_rn(cd, d.nrm_n[j]);
+        red[1] = fmax(red[1], fabs(cd * d.q_raw[j]));
+      }
+      if (!tm.template publish_sync<2, 2u>(red)) return false;
+      tm.template collect<2, 2u>(red);
+      // In γ's max a norm below 1e-4 counts as 1 (a vanishing norm carries no
+      // scale, as for δ), and the max is clamped like the other norms; taken
+      // literally with q̄ = 0 and mostly-zero P̄ columns, 1/max would grow c
+      // geometrically pass after pass.
+      double mean = red[0] / (double)n, qnv = red[1];
+      if (mean < kNormMin) mean = 1.0;
+      if (qnv < kNormMin) qnv = 1.0;
+      const double gamma = 1.0 / fmin(fmax(fmax(mean, qnv), kNormMin), kNormMax);
+      c *= gamma;
+    }
+    if (last) break;
     // δ, S ← diag(δ)S, and ‖1 − δ‖∞
-    double dev[1] = {0.0};
+    double devt[1] = {0.0};
     for (int j = et; j < n; j += nth) {
-      double dl = ruiz_delta(d.nrm_n[j]);
-      d.nrm_n[j] = 0.0;
-      d.D[j] *= dl;
-      dev[0] = fmax(dev[0], fabs(1.0 - dl));
+      const double dj = d.D[j];
+      double dl = ruiz_delta(dj * fmax(c * d.nrm_n[j], d.aty[j]));
+      d.D[j] = dj * dl;
+      devt[0] = fmax(devt[0], fabs(1.0 - dl));
     }
     for (int i = et; i < m; i += nth) {
       double dl = ruiz_delta(d.nrm_m[i]);
-      d.nrm_m[i] = 0.0;
       d.E[i] *= dl;
-      dev[0] = fmax(dev[0], fabs(1.0 - dl));
+      devt[0] = fmax(devt[0], fabs(1.0 - dl));
     }
-    if (!tm.template publish_sync<1, 1u>(dev)) return false;
-    tm.template collect<1, 1u>(dev);
+    if (!tm.template publish_sync<1, 1u>(devt)) return false;
+    tm.template collect<1, 1u>(devt);
+    dev = devt[0];
     ++passes;
-    // Cost scaling γ = 1/max{mean_j ‖P̄_:,j‖∞, ‖q̄‖∞} with the new D.
-    spmv<1, true, double, double>(
-        rows, d.kn, d.kn_ci, d.kn_raw,
-        [&](int col, double v, double* acc) {
-          if (col < n) acc[0] = fmax(acc[0], fabs(v) * d.D[col]);
-        },
-        [&](int j, double* acc) { d.nrm_n[j] = cc * d.D[j] * acc[0]; });
-    double qn[1] = {0.0};
-    for (int j = et; j < n; j += nth) qn[0] = fmax(qn[0], fabs(cc * d.D[j] * d.q_raw[j]));
-    if (!tm.template publish_sync<1, 1u>(qn)) return false;
-    tm.template collect<1, 1u>(qn);
-    double sum[1] = {0.0};
-    for (int j = tid; j < n; j += nth) {
-      sum[0] += d.nrm_n[j];
-      d.nrm_n[j] = 0.0;
-    }
-    if (!tm.template publish_sync<1, 0u>(sum)) return false;
-    tm.template collect<1, 0u>(sum);
-    // In γ's max a norm below 1e-4 counts as 1 (a vanishing norm carries no
-    // scale, as for δ), and the max is clamped like the other norms; taken
-    // literally with q̄ = 0 and mostly-zero P̄ columns, 1/max would grow c
-    // geometrically pass after pass.
-    double mean = sum[0] / (double)n, qnv = qn[0];
-    if (mean < kNormMin) mean = 1.0;
-    if (qnv < kNormMin) qnv = 1.0;
-    const double gamma = 1.0 / fmin(fmax(fmax(mean, qnv), kNormMin), kNormMax);
-    c *= gamma;
-    if (dev[0] <= P.eps_equil) break;
   }
   // Scaled data: P̄ = cDPD, Ā = EAD (in both Kn and Ā), q̄ = cDq, [El, Eu].
   foreach_entry(rows, d.kn, d.kn_ci, [&](int j, int k) {
