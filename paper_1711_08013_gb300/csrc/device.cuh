@@ -1612,7 +1612,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   const auto krows = kWide ? inner_rows(tm, d.kn) : plain;
   // this warp's first long row of w (see P1), kept where its table entries
   // cost an L2 trip per use and registers are left
-  constexpr bool kKeepRow = kWide && !Team::kCtaScope;
+  constexpr bool kKeepRow = !Team::kCtaScope;
   const int lr0 = prows.n - 1 - prows.w;
   const int lr0_row = kKeepRow && lr0 < d.kn.nlong ? d.kn.long_rows[lr0] : 0;
   const int2 lr0_range = kKeepRow && lr0 < d.kn.nlong ? d.kn.lrange[lr0] : make_int2(0, 0);

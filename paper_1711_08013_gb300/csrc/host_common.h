@@ -7,6 +7,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 #include <utility>
 #include <vector>
 
@@ -172,10 +174,16 @@ inline bool valid_csc(const osqp_csc* M, int rows, int cols, bool upper) {
   return true;
 }
 
+// No early exit and integer tests only, so that the loop vectorises (the
+// exponent is all ones exactly for Inf and NaN).
 inline bool finite_all(const double* v, int n) {
-  for (int i = 0; i < n; ++i)
-    if (!std::isfinite(v[i])) return false;
-  return true;
+  uint64_t bad = 0;
+  for (int i = 0; i < n; ++i) {
+    uint64_t b;
+    std::memcpy(&b, v + i, sizeof(b));
+    bad |= (uint64_t)((b & 0x7ff0000000000000ull) == 0x7ff0000000000000ull);
+  }
+  return bad == 0;
 }
 
 inline int check_settings(const osqp_settings& s) {

@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -244,6 +245,15 @@ __global__ void k_zero_iterates(const __grid_constant__ Dev<T> d) {
 // host side
 // ---------------------------------------------------------------------------
 
+// What a call reads back and what a launch zeroes, side by side in device
+// memory: one copy returns the scalars and the error flag, one memset readies
+// flag and barrier (a call on a small problem is bound by such steps).
+struct DevBlock {
+  Scalars sc;
+  int err, pad;
+  Barrier bar;
+};
+
 constexpr int kClusterSize = 8;  // CTAs of a cluster team (portable maximum)
 constexpr size_t kBlockPoolCap = 160 << 10;  // shared memory for a one-CTA solve's PCG vectors
 
@@ -269,10 +279,11 @@ struct osqp_solver {
   double* raw_in = nullptr;
   int *kn_src_d = nullptr, *a_src_d = nullptr;
   double *x_ws = nullptr, *y_ws = nullptr;
-  Barrier* bar = nullptr;
+  DevBlock* blk = nullptr;
+  Barrier* bar = nullptr;   // blk->bar, blk->err, blk->sc
   int* err = nullptr;
-  double* part = nullptr;
   Scalars* sc = nullptr;
+  double* part = nullptr;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   osqp_info info{};
   double rho_bar = 0.1;
@@ -377,15 +388,20 @@ cudaError_t launch_cluster(osqp_solver* s, void (*kernel)(KArgs...), Args... arg
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// error flag and barrier of the next launch zeroed
+int clear_flags(osqp_solver* s) {
+  CK(cudaMemsetAsync(s->err, 0, sizeof(DevBlock) - offsetof(DevBlock, err), s->stream));
+  return OSQP_OK;
+}
+
 template <typename T>
 int launch_scale(osqp_solver* s, int reset) {
   Dev<T>& d = dev_of<T>(s);
   if (s->use_cluster) {
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     CK(launch_cluster(s, k_scale_cluster<T>, d, s->P, s->err, s->rho_bar, reset));
   } else if (s->use_grid) {
-    CK(cudaMemsetAsync(s->bar, 0, sizeof(Barrier), s->stream));
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     double rb = s->rho_bar;
     void* args[] = {(void*)&d, (void*)&s->P, (void*)&s->bar, (void*)&s->err, (void*)&s->part,
                     (void*)&rb, (void*)&reset};
@@ -402,11 +418,10 @@ template <typename T>
 int launch_refresh(osqp_solver* s) {
   Dev<T>& d = dev_of<T>(s);
   if (s->use_cluster) {
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     CK(launch_cluster(s, k_refresh_cluster<T>, d, s->P, s->err, s->rho_bar));
   } else if (s->use_grid) {
-    CK(cudaMemsetAsync(s->bar, 0, sizeof(Barrier), s->stream));
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     double rb = s->rho_bar;
     void* args[] = {(void*)&d, (void*)&s->P, (void*)&s->bar, (void*)&s->err, (void*)&s->part,
                     (void*)&rb};
@@ -427,11 +442,10 @@ int launch_admm(osqp_solver* s) {
     CK(cudaGetLastError());
   }
   if (s->use_cluster) {
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     CK(launch_cluster(s, k_admm_cluster<T>, d, s->P, s->err));
   } else if (s->use_grid) {
-    CK(cudaMemsetAsync(s->bar, 0, sizeof(Barrier), s->stream));
-    CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
+    if (int rc = clear_flags(s)) return rc;
     void* args[] = {(void*)&d, (void*)&s->P, (void*)&s->bar, (void*)&s->err, (void*)&s->part};
     CK(cudaLaunchCooperativeKernel((const void*)k_admm_grid<T>, dim3(s->grid), dim3(kThreads), args,
                                    0, s->stream));
@@ -524,16 +538,18 @@ int scatter_raw(osqp_solver* s) {
   return OSQP_OK;
 }
 
-int read_scalars(osqp_solver* s, Scalars* out) {
-  CK(cudaMemcpyAsync(out, s->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s->stream));
+// Wait for the stream; the scalars of the last launch, and its error flag.
+int read_block(osqp_solver* s, DevBlock* out) {
+  CK(cudaMemcpyAsync(out, s->blk, offsetof(DevBlock, bar), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
-  return OSQP_OK;
+  return (s->use_grid || s->use_cluster) && out->err != kDevOk ? OSQP_ERR_DEVICE : OSQP_OK;
 }
 
-int check_device_error(osqp_solver* s) {
-  if (!s->use_grid && !s->use_cluster) return OSQP_OK;
-  int e = 0;
-  CK(cudaMemcpyAsync(&e, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+// Wait for the stream and check the error flag (one-CTA kernels have none).
+int wait_checked(osqp_solver* s) {
+  int e = kDevOk;
+  if (s->use_grid || s->use_cluster)
+    CK(cudaMemcpyAsync(&e, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   return e == kDevOk ? OSQP_OK : OSQP_ERR_DEVICE;
 }
@@ -676,10 +692,8 @@ size_t arena_bytes_for(osqp_solver* s, size_t part_doubles) {
   A.take<int>(s->a_s.npos);
   A.take<double>(s->n);
   A.take<double>(s->m);
-  A.take<Barrier>(1);
-  A.take<int>(1);
   A.take<double>(part_doubles);
-  A.take<Scalars>(1);
+  A.take<DevBlock>(1);
   return A.off + 256;
 }
 
@@ -693,10 +707,11 @@ int carve_and_upload(osqp_solver* s, size_t part_doubles) {
   s->a_src_d = A.take<int>(s->a_s.npos);
   s->x_ws = A.take<double>(s->n);
   s->y_ws = A.take<double>(s->m);
-  s->bar = A.take<Barrier>(1);
-  s->err = A.take<int>(1);
   s->part = A.take<double>(part_doubles);
-  s->sc = A.take<Scalars>(1);
+  s->blk = A.take<DevBlock>(1);
+  s->bar = &s->blk->bar;
+  s->err = &s->blk->err;
+  s->sc = &s->blk->sc;
   d.sc = s->sc;
   auto up = [&](void* dst, const void* src, size_t bytes) -> cudaError_t {
     if (bytes == 0) return cudaSuccess;
@@ -719,7 +734,7 @@ int carve_and_upload(osqp_solver* s, size_t part_doubles) {
     if (!h.lrange.empty())
       CK(cudaMemsetAsync(S.ccount, 0, h.lrange.size() * sizeof(unsigned), s->stream));
   }
-  CK(cudaMemsetAsync(s->sc, 0, sizeof(Scalars), s->stream));
+  CK(cudaMemsetAsync(s->blk, 0, sizeof(DevBlock), s->stream));
   return OSQP_OK;
 }
 
@@ -951,8 +966,7 @@ int32_t osqp_setup(osqp_solver** out, const osqp_csc* P, const double* q, const 
   if (cudaEventRecord(s->ev[0], s->stream) != cudaSuccess) return fail(OSQP_ERR_CUDA);
   if ((rc = do_scale(s, 1))) return fail(rc);
   if (cudaEventRecord(s->ev[1], s->stream) != cudaSuccess) return fail(OSQP_ERR_CUDA);
-  if (cudaStreamSynchronize(s->stream) != cudaSuccess) return fail(OSQP_ERR_CUDA);
-  if ((rc = check_device_error(s))) return fail(rc);
+  if ((rc = wait_checked(s))) return fail(rc);
   s->info.setup_time = elapsed_s(s->ev[0], s->ev[1]);
   s->info.launch = s->use_cluster ? 3 : (s->use_grid ? 2 : 1);
   *out = s;
@@ -970,10 +984,9 @@ int32_t osqp_solve_async(osqp_solver* s) {
 }
 
 static int32_t refresh_info(osqp_solver* s) {
-  Scalars sc;
-  int rc;
-  if ((rc = read_scalars(s, &sc))) return rc;
-  if ((rc = check_device_error(s))) return rc;
+  DevBlock blk;
+  if (int rc = read_block(s, &blk)) return rc;
+  const Scalars& sc = blk.sc;
   s->info.status = sc.status;
   s->info.iter = sc.iter;
   s->info.pcg_iters = sc.pcg_iters;
@@ -1001,12 +1014,12 @@ int32_t osqp_update_vectors(osqp_solver* s, const double* q, const double* l, co
   if (q && !finite_all(q, s->n)) return OSQP_ERR_NONFINITE;
   // Check l ≤ u against the stored value of whichever side is not replaced.
   if (l || u) {
-    std::vector<double> lh(s->m), uh(s->m);
+    std::vector<double> lh(l ? 0 : s->m), uh(u ? 0 : s->m);
     double *kn_raw, *a_raw, *qd, *ld, *ud;
     get_raw(s, &kn_raw, &a_raw, &qd, &ld, &ud);
     if (!l && s->m) CK(cudaMemcpyAsync(lh.data(), ld, sizeof(double) * s->m, cudaMemcpyDeviceToHost, s->stream));
     if (!u && s->m) CK(cudaMemcpyAsync(uh.data(), ud, sizeof(double) * s->m, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaStreamSynchronize(s->stream));
+    if (!l || !u) CK(cudaStreamSynchronize(s->stream));
     const double* L = l ? l : lh.data();
     const double* U = u ? u : uh.data();
     for (int i = 0; i < s->m; ++i) {
@@ -1017,8 +1030,7 @@ int32_t osqp_update_vectors(osqp_solver* s, const double* q, const double* l, co
   int rc = upload_vectors(s, q, l, u, cudaMemcpyHostToDevice);
   if (rc) return rc;
   if ((rc = do_refresh(s))) return rc;
-  CK(cudaStreamSynchronize(s->stream));
-  return check_device_error(s);
+  return wait_checked(s);
 }
 
 int32_t osqp_update_matrices(osqp_solver* s, const double* Pv, const double* Av) {
@@ -1035,9 +1047,9 @@ int32_t osqp_update_matrices(osqp_solver* s, const double* Pv, const double* Av)
   CK(cudaEventRecord(s->ev[0], s->stream));
   if ((rc = do_scale(s, 0))) return rc;
   CK(cudaEventRecord(s->ev[1], s->stream));
-  CK(cudaStreamSynchronize(s->stream));
+  rc = wait_checked(s);
   s->info.setup_time = elapsed_s(s->ev[0], s->ev[1]);
-  return check_device_error(s);
+  return rc;
 }
 
 static int32_t load_data(osqp_solver* s, const double* Pv, const double* q, const double* Av,
@@ -1070,8 +1082,7 @@ int32_t osqp_update_rho(osqp_solver* s, double rho_bar) {
   s->rho_bar = rho_bar;
   int rc = do_refresh(s);
   if (rc) return rc;
-  CK(cudaStreamSynchronize(s->stream));
-  return check_device_error(s);
+  return wait_checked(s);
 }
 
 int32_t osqp_warm_start(osqp_solver* s, const double* x, const double* y) {
@@ -1094,12 +1105,13 @@ int32_t osqp_get_solution(osqp_solver* s, double* x, double* y, double* z, osqp_
     CK(cudaMemcpyAsync(y, out_y(s), sizeof(double) * s->m, cudaMemcpyDeviceToHost, s->stream));
   if (z && s->m)
     CK(cudaMemcpyAsync(z, out_z(s), sizeof(double) * s->m, cudaMemcpyDeviceToHost, s->stream));
-  CK(cudaStreamSynchronize(s->stream));
-  if (info) {
+  if (info) {  // waits for the stream
     int rc = refresh_info(s);
     if (rc) return rc;
     *info = s->info;
+    return OSQP_OK;
   }
+  CK(cudaStreamSynchronize(s->stream));
   return OSQP_OK;
 }
 
