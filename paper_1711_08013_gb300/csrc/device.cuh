@@ -1718,6 +1718,10 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     rd_bar = res[1];
   }
   bool have_check = rp_bar > 0.0 && rd_bar > 0.0;
+  // the tolerance needs ‖b‖∞ itself until the next check; largest column sum
+  // of |Ā| (−1: not formed yet) — see R
+  bool exact_b = false;
+  double colsum = -1.0;
 
   for (k = 1; k <= P.max_iter; ++k) {
     // --- R: initial PCG residual r⁰ = b − Kx̃ and b = σx − q̄ + Āᵀ(Rz − y),
@@ -1725,27 +1729,69 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // from FP64 vectors with FP64 accumulation in both modes, so that in the
     // FP32 mode every ADMM iteration restarts PCG from an accurate residual
     // (mixed-precision iterative refinement of the linear solve).
+    //
+    // b itself only enters the PCG tolerance, through the floor τ‖b‖∞ (and
+    // before the first check through ‖b‖∞ alone).  Its product is a third of
+    // the stage's FP64 instructions, which bound it, so after a check b is
+    // left out while the bound ‖b‖∞ ≤ ‖σx − q̄‖∞ + max_j Σ_i|Ā_ij|·‖Rz − y‖∞
+    // shows that the floor is not the largest term: the tolerance is then the
+    // same number.  Otherwise the stage runs once more with b, and keeps it
+    // until the next check.  FP64 mode only: in the FP32-mixed one-CTA kernel
+    // the second form of the stage cost the products their registers (MPC
+    // batch 126.8 -> 186.7 ms).
+    if (kWide && have_check && colsum < 0.0) {
+      double cs[1] = {0.0};
+      auto row = [&](int, double* acc) { cs[0] = fmax(cs[0], acc[0]); };
+      spmv<1, false, double, T>(
+          rows, d.kn, kn_ci, kn_v,
+          [&](int col, T v, double* acc) {
+            if (col >= n) acc[0] += fabs((double)v);
+          },
+          row);
+      if (!tm.template publish_sync<1, 1u>(cs)) return false;
+      tm.template collect<1, 1u>(cs);
+      colsum = cs[0];
+    }
+    bool with_b = !kWide || !have_check || exact_b;
+    bool done;
+    for (;;) {
     {
       T* __restrict__ r = rbuf(cur);
       T* __restrict__ u0 = ubuf(cur);
-      spmv<2, false, double, T>(
-          rows, d.kn, kn_ci, kn_v,
-          [&](int col, T v, double* acc) {
-            const double vv = (double)v;
-            if (col < n) {
-              acc[0] -= vv * xt[col];
-            } else {
-              acc[0] += vv * um[col - n];
-              acc[1] += vv * wm[col - n];
-            }
-          },
-          [&](int j, double* acc) {
-            const double bj = sigma * x[j] - d.q[j];
-            const T rj = T(bj - sigma * xt[j] + acc[0]);
-            r[j] = rj;
-            u0[j] = rj * dinv[j];  // here, so that A0 gathers u instead of r and M⁻¹
-            bv[j] = T(bj + acc[1]);
-          });
+      auto store = [&](int j, double bj, double acc, double b) {
+        const T rj = T(bj - sigma * xt[j] + acc);
+        r[j] = rj;
+        u0[j] = rj * dinv[j];  // here, so that A0 gathers u instead of r and M⁻¹
+        bv[j] = T(b);
+      };
+      if (!kWide || with_b)
+        spmv<2, false, double, T>(
+            rows, d.kn, kn_ci, kn_v,
+            [&](int col, T v, double* acc) {
+              const double vv = (double)v;
+              if (col < n) {
+                acc[0] -= vv * xt[col];
+              } else {
+                acc[0] += vv * um[col - n];
+                acc[1] += vv * wm[col - n];
+              }
+            },
+            [&](int j, double* acc) {
+              const double bj = sigma * x[j] - d.q[j];
+              store(j, bj, acc[0], bj + acc[1]);
+            });
+      else
+        spmv<1, false, double, T>(
+            rows, d.kn, kn_ci, kn_v,
+            [&](int col, T v, double* acc) {
+              const double vv = (double)v;
+              if (col < n) acc[0] -= vv * xt[col];
+              else acc[0] += vv * um[col - n];
+            },
+            [&](int j, double* acc) {
+              const double bj = sigma * x[j] - d.q[j];
+              store(j, bj, acc[0], bj);
+            });
     }
     if (!tm.sync()) return false;
 
@@ -1754,7 +1800,8 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // and computes t = RĀu with u formed on the fly, and one stage that forms
     // w = Ku and the two inner products (r,u), (w,u).  r, s, w and t are
     // double-buffered so that gathers never see a vector being rewritten.
-    // --- A0: t = RĀu with the u = M⁻¹r that R left; (r,u), ‖r‖∞, ‖b‖∞
+    // --- A0: t = RĀu with the u = M⁻¹r that R left; (r,u), ‖r‖∞, ‖b‖∞ (or half
+    // its bound)
     T red3t[3];
     {
       const T* __restrict__ r = rbuf(cur);
@@ -1767,6 +1814,11 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         a1 = fmax(a1, fabs(rj));
         a2 = fmax(a2, fabs(bv[j]));
       }
+      if (kWide && !with_b) {
+        double w = 0.0;
+        for (int i = et; i < m; i += nth) w = fmax(w, fabs(wm[i]));
+        a2 = fmax(a2, T(colsum * w));
+      }
       red3t[0] = a0;
       red3t[1] = a1;
       red3t[2] = a2;
@@ -1777,17 +1829,29 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     }
     if (!tm.template reduce<3, 6u, true, kF32>(red3t, [&](const double (&red3)[3]) {
           // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
-          const double bnorm = red3[2];
-          const double tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
-                                  have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
-                                             : 0.1 * P.pcg_kappa * bnorm);
+          double tol;
+          int flag = 0;
+          if (!kWide || with_b) {
+            const double bnorm = red3[2];
+            tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
+                       have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
+                                  : 0.1 * P.pcg_kappa * bnorm);
+          } else {
+            // both terms of the bound are at most red3[2] (rounded to T)
+            tol = fmax(P.pcg_reduce * red3[1], P.pcg_kappa * fmin(rp_bar, rd_bar));
+            if (!(P.pcg_floor * (2.02 * red3[2]) <= tol)) flag = 2;
+          }
           scal[0] = red3[0];  // γ = (r, M⁻¹r)
           scal[3] = tol;
           if (kF32) *ftol = (float)tol;
-          *sflag = !(red3[1] > tol);
+          *sflag = flag ? flag : !(red3[1] > tol);
         }))
       return false;
-    bool done = *sflag != 0;
+    const int flag = *sflag;
+    done = flag != 0;
+    if (!kWide || flag != 2) break;
+    exact_b = with_b = true;
+    }
     if constexpr (kF32) {
       cg_g = ff{fmir[0], fmir[1]};
       cg_tol = *ftol;
@@ -2138,6 +2202,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     rp_bar = R[3];
     rd_bar = R[10];
     have_check = true;
+    exact_b = false;
     // ρ̄ adaptation (§5.2) in scaled norms; the Jacobi diagonal is rebuilt
     // on the device in place of a refactorisation.
     if (P.adaptive_rho && rho_updates < P.max_rho_updates && k < P.max_iter) {

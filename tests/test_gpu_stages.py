@@ -1,5 +1,5 @@
-"""Numbering of the whole-GPU team's warps: the rule that picks it for the
-inner-product products changes at half as many slices as warps."""
+"""Stages of the solve at the edges of their rules: the numbering of the
+whole-GPU team's warps, the tolerance without ‖b‖∞, the scaling passes."""
 import numpy as np
 import pytest
 
@@ -47,3 +47,29 @@ def test_step_parity_on_the_grid(oracle_mod, name):
         g = s.solve()
     assert g.iter == 7
     assert rel_err(g.x, o.x) <= 1e-8 and rel_err(g.z, o.z) <= 1e-8 and rel_err(g.y, o.y) <= 1e-8
+
+
+@pytest.mark.parametrize("launch", [1, 2, 3], ids=["block", "grid", "cluster"])
+@pytest.mark.parametrize("name", ["lasso", "random"])
+def test_tolerance_floor_is_kept_when_b_is_left_out(name, launch):
+    """A PCG floor of 10³‖b‖∞ is above the first residual (x̃ = 0, r⁰ = b) in
+    every iteration, before and after checks: no PCG iteration may run,
+    whether ‖b‖∞ was formed or only bounded."""
+    qp = pb.lasso(5, seed=6) if name == "lasso" else pb.random_qp(20, 90, seed=7)
+    with Solver(qp, launch=launch, pcg_tol_floor=1e3, check_interval=5, max_iter=60,
+                eps_abs=1e-9, eps_rel=1e-9, eps_pinf=1e-300, eps_dinf=1e-300) as s:
+        g = s.solve()
+    assert g.iter == 60 and g.pcg_iters == 0
+
+
+@pytest.mark.parametrize("launch", [1, 2], ids=["block", "grid"])
+@pytest.mark.parametrize("passes", [0, 1, 2, 10])
+def test_scaling_after_a_number_of_passes(oracle_mod, passes, launch):
+    """D, E and c after the last pass, whose cost factor needs one more product
+    than its norms: the oracle's to 1e-12."""
+    qp = pb.portfolio(3, seed=5)
+    want = oracle_mod.ruiz(qp.P_full(), qp.q, qp.A, qp.l, qp.u, scaling_iters=passes)
+    with Solver(qp, launch=launch, scaling_iters=passes) as s:
+        D, E, c, _ = s.scaling()
+    assert rel_err(D, want["D"]) <= 1e-12 and rel_err(E, want["E"]) <= 1e-12
+    assert abs(c - want["c"]) <= 1e-12 * want["c"]
