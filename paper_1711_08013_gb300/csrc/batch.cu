@@ -78,7 +78,7 @@ __device__ void batch_solve_one(Team& tm, const Dev<T>& d, const Params& P, int 
 // As batch_solve_one, with the PCG vectors in the CTA's shared memory (one
 // CTA per problem; the problem's vectors fit in `pool`).
 template <typename T>
-__device__ void batch_solve_one_smem(BlockTeam& tm, const Dev<T>& d, const Params& P, int md,
+__device__ void batch_solve_one_smem(FullTeam& tm, const Dev<T>& d, const Params& P, int md,
                                      Dev<T>& sd, unsigned char* pool, bool with_mat) {
   const double rho_bar = d.sc->rho_bar;
   if (md & kModeScale) {
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   __shared__ int sidx;
   __shared__ Dev<T> sdev;
   extern __shared__ __align__(16) unsigned char pool[];
-  BlockTeam tm{sm};
+  FullTeam tm{{sm}};
   for (;;) {
     if (threadIdx.x == 0) sidx = atomicAdd(queue, 1);
     __syncthreads();

@@ -407,6 +407,7 @@ __device__ __forceinline__ double ld_partial(const double* p) {
 
 struct GridTeam {
   static constexpr bool kCtaScope = false;  // products span CTAs
+  static constexpr bool kBoundB = true;  // stage R may leave b out (admm_stage)
   Barrier* bar;
   int* err;
   double* part;  // [2][kMaxRed][gridDim.x]: a slot's partials are contiguous
@@ -670,6 +671,7 @@ __device__ __forceinline__ void cluster_sync_all() {
 // cluster's partials in rank order, so all CTAs hold identical values.
 struct ClusterTeam {
   static constexpr bool kCtaScope = false;
+  static constexpr bool kBoundB = true;
   static constexpr unsigned int kBarrierPoison = 0x80000000u;
   double* sm;
   double* cpart;  // [2][kMaxRed] this CTA's published block results
@@ -780,6 +782,7 @@ struct ClusterTeam {
 
 struct BlockTeam {
   static constexpr bool kCtaScope = true;  // every warp of a product is in this CTA
+  static constexpr bool kBoundB = true;
   double* sm;
   __device__ int nthreads() const { return blockDim.x; }
   __device__ int tid() const { return threadIdx.x; }
@@ -830,6 +833,13 @@ struct BlockTeam {
 };
 
 // A plain (non-cooperative) launch as a traversal team: no barriers.
+// The one-CTA team of the kernels that also build or stage the problem: their
+// stage R always forms b.  With the second form of the stage the batch kernel
+// was slower in both modes (608 MPC QPs, FP64: 313 -> 362 ms).
+struct FullTeam : BlockTeam {
+  static constexpr bool kBoundB = false;
+};
+
 struct PlainTeam {
   static constexpr bool kCtaScope = false;
   __device__ int nthreads() const { return gridDim.x * blockDim.x; }
@@ -1615,6 +1625,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   // FP32-mixed: 42.8 ms plain, 44.5 ms spread)
   constexpr bool kWide = sizeof(T) == sizeof(double);
   const Warps<Team::kCtaScope> plain{tm.warp(), tm.nwarps()};
+  constexpr bool kBoundB = kWide && Team::kBoundB;  // see R
   const auto prows = kWide ? rows : plain;
   const int pt = kWide ? et : tid;
   const auto krows = kWide ? inner_rows(tm, d.kn) : plain;
@@ -1751,7 +1762,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // solve 2 %, but the batch kernel lost a third of its speed at the same
     // registers and spills, as a second form of the stage (608 MPC QPs 126.8
     // -> 186.7 ms) and as a predicate in the first (129.3 -> 188.2 ms).
-    if (kWide && have_check && colsum < 0.0) {
+    if (kBoundB && have_check && colsum < 0.0) {
       double cs[1] = {0.0};
       auto row = [&](int, double* acc) { cs[0] = fmax(cs[0], acc[0]); };
       spmv<1, false, double, T>(
@@ -1764,7 +1775,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       tm.template collect<1, 1u>(cs);
       colsum = cs[0];
     }
-    bool with_b = !kWide || !have_check || exact_b;
+    bool with_b = !kBoundB || !have_check || exact_b;
     bool done;
     for (;;) {
     {
@@ -1779,7 +1790,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         u0[j] = rj * dinv[j];
         bv[j] = T(b);
       };
-      if (!kWide || with_b)
+      if (!kBoundB || with_b)
         spmv<2, false, double, T>(
             rows, d.kn, kn_ci, kn_v,
             [&](int col, T v, double* acc) {
@@ -1829,7 +1840,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         a1 = fmax(a1, fabs(rj));
         a2 = fmax(a2, fabs(bv[j]));
       }
-      if (kWide && !with_b) {
+      if (kBoundB && !with_b) {
         double w = 0.0;
         for (int i = et; i < m; i += nth) w = fmax(w, fabs(wm[i]));
         a2 = fmax(a2, T(colsum * w));
@@ -1846,7 +1857,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
           double tol;
           int flag = 0;
-          if (!kWide || with_b) {
+          if (!kBoundB || with_b) {
             const double bnorm = red3[2];
             tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
                        have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
@@ -1864,7 +1875,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       return false;
     const int flag = *sflag;
     done = flag != 0;
-    if (!kWide || flag != 2) break;
+    if (!kBoundB || flag != 2) break;
     exact_b = with_b = true;
     }
     if constexpr (kF32) {

@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kThreads) k_noalloc(NaInput in, const __grid_c
     if (tid == 0) d.sc->dev_error = sp.err[0];
     return;
   }
-  BlockTeam tm{sm};
+  FullTeam tm{{sm}};
   if (!scale_stage(tm, d, P, rho0, true)) return;
   admm_stage(tm, d, P);
 }
