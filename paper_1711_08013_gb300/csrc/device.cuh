@@ -1596,21 +1596,6 @@ __device__ void stage_out(const Dev<T>& d, const Dev<T>& sd) {
   __syncthreads();
 }
 
-// Numbering of the products that also add up the inner product (w, u) per
-// thread (the terms of one CTA share a partial sum).  The spread numbering
-// where Kn has no more chunks and no more slices than half the warps: there
-// the plain one would leave more than half of the SMs without work, and every
-// thread adds at most two terms.  Above that the sums stay grouped as the
-// rows are dealt.  The line measured on both sides: the Kn product of a
-// 500-variable QP (32 of 152 SMs busy in the plain numbering) is below it; its
-// solve took 12.4 -> 9.6 ms with all stages spread.
-template <class Team>
-__device__ __forceinline__ Warps<Team::kCtaScope> inner_rows(const Team& tm, const Sched& S) {
-  const int half = tm.nwarps() / 2;
-  if (S.nslices <= half && S.nchunks <= half) return tm.spread();
-  return {tm.warp(), tm.nwarps()};
-}
-
 // ---------------------------------------------------------------------------
 // Stage 2: Algorithm 1 with the indirect linear solve of §3.1.
 // ---------------------------------------------------------------------------
@@ -1624,11 +1609,13 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   // pipe, and few SMs share the gathered lines of u better than many (Lasso
   // FP32-mixed: 42.8 ms plain, 44.5 ms spread)
   constexpr bool kWide = sizeof(T) == sizeof(double);
+  // the products that also add up (w, u) keep the plain numbering in both
+  // modes: a CTA's rows share a partial sum, and regrouping it moves the sum
+  // by a rounding that a long CG run amplifies into other iterates
   const Warps<Team::kCtaScope> plain{tm.warp(), tm.nwarps()};
   constexpr bool kBoundB = kWide && Team::kBoundB;  // see R
   const auto prows = kWide ? rows : plain;
   const int pt = kWide ? et : tid;
-  const auto krows = kWide ? inner_rows(tm, d.kn) : plain;
   // this warp's first long row of w (see P1), kept where its table entries
   // cost an L2 trip per use and registers are left
   constexpr bool kKeepRow = !Team::kCtaScope;
@@ -1890,7 +1877,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       const T* __restrict__ u = ut;
       // long rows of w stay as chunk partials: P1, the only reader, sums them
       spmv<1, false, T, T>(
-          krows, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
+          plain, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
           [&](int j, T* acc) {
             const T wj = sigT * u[j] + acc[0];
             w[j] = wj;
@@ -2012,7 +1999,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           g2 = fmax(g2, fabs(rj));
         }
         spmv<1, false, T, T>(
-            krows, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
+            plain, d.kn, kn_ci, kn_v, [&](int col, T v, T* acc) { acc[0] += v * ut[col]; },
             [&](int j, T* acc) {
               const T wj = sigT * u[j] + acc[0];
               wn[j] = wj;

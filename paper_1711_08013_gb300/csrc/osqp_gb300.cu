@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads)
   GridTeam tm{bar, err, part, sm, timeout_ns, 0, 0u};
   // the numbering of the solve's own product (see admm_stage)
   Warps<false> numbering{tm.warp(), tm.nwarps()};
-  if constexpr (sizeof(T) == sizeof(double)) numbering = KN ? inner_rows(tm, S) : tm.spread();
+  if constexpr (!KN && sizeof(T) == sizeof(double)) numbering = tm.spread();
   for (int r = 0; r < reps; ++r) {
     T acc1 = T(0);
     if constexpr (KN) {
