@@ -1622,6 +1622,8 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
   const int lr0 = prows.n - 1 - prows.w;
   const int lr0_row = kKeepRow && lr0 < d.kn.nlong ? d.kn.long_rows[lr0] : 0;
   const int2 lr0_range = kKeepRow && lr0 < d.kn.nlong ? d.kn.lrange[lr0] : make_int2(0, 0);
+  // … and the kind of this thread's first row, which P1 needs before the row's inputs
+  const bool short0 = kKeepRow && pt < n && d.kn.lidx[pt] < 0;
   const double sigma = P.sigma, alpha = P.alpha;
   const T sigT = T(sigma);
   const double c = d.sc->c;
@@ -1950,11 +1952,10 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
         // chains run on different warps
         const bool lazy_w = d.kn.nlong > 0;
         for (int j = pt; j < n; j += nth) {
-          // (the row kind is fetched beside the inputs, not before them)
-          const bool mine = !lazy_w || d.kn.lidx[j] < 0;
-          const T wj = wc[j];
-          const In e = fetch(j);
-          if (mine) upd(j, wj, e);
+          // a long row's element is its warp's alone: w_j was not stored, and
+          // p_j and δx̃_j are rewritten below while other threads are here
+          const bool mine = !lazy_w || (kKeepRow && j == pt ? short0 : d.kn.lidx[j] < 0);
+          if (mine) upd(j, wc[j], fetch(j));
         }
         for (int lr = prows.n - 1 - prows.w; lr < d.kn.nlong; lr += prows.n) {
           // place of the row known in advance; its inputs travel with the
@@ -1962,9 +1963,11 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
           const bool kept = kKeepRow && lr == lr0;
           const int j = kept ? lr0_row : d.kn.long_rows[lr];
           const int2 rg = kept ? lr0_range : d.kn.lrange[lr];
-          const In e = fetch(j);
+          const bool lane0 = (threadIdx.x & 31) == 0;  // the lane that rewrites p_j and δx̃_j
+          In e{};
+          if (lane0) e = fetch(j);
           const T sum = warp_long_sum<T>(d.kn, rg, 0);
-          if ((threadIdx.x & 31) == 0) upd(j, sigT * e.u + sum, e);
+          if (lane0) upd(j, sigT * e.u + sum, e);
         }
         for (int i = pt; i < m; i += nth) {
           const T ti = rho_invT[i] * tc[i];

@@ -25,11 +25,28 @@ from paper_1711_08013_gb300.solver import Solver  # noqa: E402
 CTA_WARPS = 16
 
 
+def long_row_qp():
+    """One variable in all 256 constraints and in a dense row of P: its row of
+    [P Aᵀ] has 276 nonzeros, two chunks."""
+    n, m = 20, 256
+    rng = np.random.default_rng(11)
+    M = np.diag(2.0 + rng.random(n))
+    M[0, 1:] = 0.05 * rng.standard_normal(n - 1)
+    rows = np.arange(m)
+    A = sp.csc_matrix((rng.standard_normal(2 * m),
+                       (np.concatenate([rows, rows]),
+                        np.concatenate([np.zeros(m, int), 1 + rows % (n - 1)]))), shape=(m, n))
+    mid = A @ rng.standard_normal(n)
+    return pb._finish("long_row", M + M.T, rng.standard_normal(n), A, mid - 0.3 * rng.random(m),
+                      mid + 0.3 * rng.random(m))
+
+
 PROBLEMS = {
     "all_warps": lambda: pb.mpc_paper(4, T=10, seed=1),  # 16 slices of Kn
     "nine_warps": lambda: pb.mpc_paper(3, T=8, seed=2),
     "whole_warp_rows": lambda: pb.random_qp(10, 100, seed=3),
     "quarter_warp_rows": lambda: pb.svm(1, seed=4),
+    "long_row": long_row_qp,
 }
 
 
@@ -52,6 +69,7 @@ def test_teams_give_the_bits_of_one_cta(name, launch):
     for M in (sp.hstack([qp.P_full(), qp.A.T]).tocsr(), qp.A.tocsr()):
         part = partition(M, CTA_WARPS)
         assert part == partition(M, warps) and part[2] <= CTA_WARPS and part[5] <= CTA_WARPS
+        assert part[4] == (1 if name == "long_row" and M.shape[0] == qp.n else 0)
     res = []
     for team in (1, launch):
         with Solver(qp, launch=team, autotune=0, max_iter=100, eps_abs=1e-12, eps_rel=0.0) as s:
