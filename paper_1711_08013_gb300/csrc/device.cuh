@@ -95,6 +95,9 @@ struct Scalars {
   // continues from the current iterates takes its first PCG tolerance from
   // them (0: no check since the iterates were last reset)
   double rp_last, rd_last;
+  // largest column sum of the scaled |Ā|, formed by the first solve that wants
+  // it (admm_stage, R); −1: not formed since the matrices were scaled
+  double colsum;
   int polished, pad2;  // 1 polished, -1 rejected, 0 not run (§4)
 };
 
@@ -1251,6 +1254,7 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
   if (tm.leader()) {
     d.sc->c = c;
     d.sc->ruiz_passes = passes;
+    d.sc->colsum = -1.0;
     d.sc->rho_bar = rho_bar;
   }
   return tm.sync();
@@ -1726,10 +1730,10 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     rd_bar = res[1];
   }
   bool have_check = rp_bar > 0.0 && rd_bar > 0.0;
-  // the tolerance needs ‖b‖∞ itself until the next check; largest column sum
-  // of |Ā| (−1: not formed yet) — see R
-  bool exact_b = false;
-  double colsum = -1.0;
+  // the tolerance needs ‖b‖∞ itself (see R): from the start where the floor is
+  // all there is to it
+  bool exact_b = P.pcg_floor > 0.0 && !(P.pcg_kappa > 0.0);
+  double colsum = d.sc->colsum;
 
   for (k = 1; k <= P.max_iter; ++k) {
     // --- R: initial PCG residual r⁰ = b − Kx̃ and b = σx − q̄ + Āᵀ(Rz − y),
@@ -1743,15 +1747,17 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // the stage's FP64 instructions, which bound it, so after a check b is
     // left out while the bound ‖b‖∞ ≤ ‖σx − q̄‖∞ + max_j Σ_i|Ā_ij|·‖Rz − y‖∞
     // shows that the floor is not the largest term: the tolerance is then the
-    // same number.  Otherwise the stage runs once more with b, and keeps it
-    // until the next check.  Measured in FP64, as the gain over a solver with
+    // same number.  Otherwise the stage runs once more with b, and keeps it for
+    // the rest of the solve: residuals mostly fall from check to check, so a
+    // floor that binds stays binding (trying again after every check cost a
+    // solve with check_interval = 1 a second R and A0 in each iteration).  Measured in FP64, as the gain over a solver with
     // none of these stages' forms, before -> after: random QP n = 50 1.06× ->
     // 1.12× (7.3 -> 6.6 ms in all), MPC step 1.18× -> 1.19×.  FP64 mode only:
     // in FP32-mixed mode the whole-GPU Lasso gains 1 % and a one-CTA
     // solve 2 %, but the batch kernel lost a third of its speed at the same
     // registers and spills, as a second form of the stage (608 MPC QPs 126.8
     // -> 186.7 ms) and as a predicate in the first (129.3 -> 188.2 ms).
-    if (kBoundB && have_check && colsum < 0.0) {
+    if (kBoundB && have_check && !exact_b && colsum < 0.0) {
       double cs[1] = {0.0};
       auto row = [&](int, double* acc) { cs[0] = fmax(cs[0], acc[0]); };
       spmv<1, false, double, T>(
@@ -1763,6 +1769,7 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
       if (!tm.template publish_sync<1, 1u>(cs)) return false;
       tm.template collect<1, 1u>(cs);
       colsum = cs[0];
+      if (tm.leader()) d.sc->colsum = colsum;
     }
     bool with_b = !kBoundB || !have_check || exact_b;
     bool done;
@@ -2217,7 +2224,6 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     rp_bar = R[3];
     rd_bar = R[10];
     have_check = true;
-    exact_b = false;
     // ρ̄ adaptation (§5.2) in scaled norms; the Jacobi diagonal is rebuilt
     // on the device in place of a refactorisation.
     if (P.adaptive_rho && rho_updates < P.max_rho_updates && k < P.max_iter) {
