@@ -28,7 +28,7 @@ using namespace osqpgb::host;
 
 namespace {
 
-constexpr int kBatchThreads = 512;
+constexpr int kBatchThreads = kThreads;  // block_reduce stages one value per thread of kThreads
 constexpr long long kBatchWarps = kBatchThreads / 32;
 constexpr int kBatchCluster = 8;      // CTAs of a heavy-problem cluster
 constexpr int kMaxHeavyClusters = 4;  // clusters a launch may take for heavy problems

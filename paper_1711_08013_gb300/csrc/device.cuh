@@ -189,6 +189,7 @@ template <int K, unsigned MAXMASK>
 __device__ __forceinline__ void block_reduce(const double (&v)[K], double* sm) {
   static_assert(K <= kMaxRed, "too many reduction slots");
   if constexpr (K <= kMaxSumSlots) {
+    static_assert(kThreads == 16 * 32, "a lane adds 16 staged values");
     // one warp per slot, the maxima beside the sums (a max slot that every
     // warp first combined by shuffles cost about 250 cycles before the
     // barrier and as much again on the warp that also adds a sum)
