@@ -141,11 +141,10 @@ __global__ void __launch_bounds__(kThreads) k_barrier_probe(Barrier* bar, int* e
 }
 
 // Autotuner of a single problem's row partition on the grid team: `reps`
-// products shaped like the PCG loop's (Alg. 1, step 3), each followed by a
-// grid reduction and barrier as in the solve.  KN: w = σu + Kn u with long
-// rows left as chunk partials and the inner product (w, u) reduced; else
-// t = ρ ∘ Ā (D⁻¹ r), the preconditioned residual gathered on the fly.  x and
-// x2 hold ones (x: the gathered vector, x2: the diagonal factor).
+// products shaped like the PCG loop's (Alg. 1, step 3).  KN: w = σu + Kn u with
+// long rows left as chunk partials and the inner product (w, u) reduced by the
+// solve's one-warp reduction; else t = ρ ∘ Ā u and the barrier that follows
+// it.  x and x2 hold ones (x: the gathered vector, x2: the diagonal factor).
 template <typename T, bool KN>
 __global__ void __launch_bounds__(kThreads)
     k_tune_grid(const __grid_constant__ Sched S, const int* __restrict__ ci,
@@ -158,8 +157,8 @@ __global__ void __launch_bounds__(kThreads)
   Warps<false> numbering{tm.warp(), tm.nwarps()};
   if constexpr (!KN && sizeof(T) == sizeof(double)) numbering = tm.spread();
   for (int r = 0; r < reps; ++r) {
-    T acc1 = T(0);
     if constexpr (KN) {
+      T acc1 = T(0);
       spmv<1, false, T, T>(
           numbering, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * x[col]; },
           [&](int j, T* acc) {
@@ -169,19 +168,14 @@ __global__ void __launch_bounds__(kThreads)
           },
           [&](int j, int first, T* acc) { acc1 += (acc[0] + (first ? x2[j] : T(0))) * x[j]; },
           NoLong{}, LazyTag{});
+      const T red_t[1] = {acc1};
+      if (!tm.template reduce<1, 0u>(red_t, [](const double (&)[1]) {})) return;
     } else {
       spmv<1, false, T, T>(
-          numbering, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * (x[col] * x2[col]); },
-          [&](int i, T* acc) {
-            y[i] = x2[i] * acc[0];
-            acc1 += y[i];
-          });
+          numbering, S, ci, va, [&](int col, T v, T* acc) { acc[0] += v * x[col]; },
+          [&](int i, T* acc) { y[i] = x2[i] * acc[0]; });
+      if (!tm.sync()) return;
     }
-    const T red_t[1] = {acc1};
-    tm.template publish<1, 0u>(red_t);
-    if (!tm.sync()) return;
-    double red[1];
-    tm.template collect<1, 0u>(red);
   }
 }
 
