@@ -352,12 +352,13 @@ int32_t osqp_diag_schedule(osqp_solver* s, int32_t* groups, double* ms);
 
 /* Diagnostic of the bounded grid barrier that every multi-CTA solve relies
  * on (the paper has no counterpart).  Launches four cooperative CTAs on the
- * current device, one of which never arrives at the barrier; the others must
- * give up after timeout_s seconds (0 < timeout_s ≤ 10), record the timeout
- * and return, leaving the context usable.  Returns OSQP_OK when exactly
- * that happened, OSQP_ERR_DEVICE if the barrier did not report the timeout,
- * OSQP_ERR_ARG for a bad timeout, OSQP_ERR_CUDA on a CUDA error.  Allocates
- * and frees a few bytes of device memory; synchronises the device. */
+ * current device, one of which never arrives at the barrier, then the same in
+ * a reduction over the CTAs; each time the others must give up after timeout_s
+ * seconds (0 < timeout_s ≤ 10), record the timeout and return, leaving the
+ * context usable.  Returns OSQP_OK when exactly that happened both times,
+ * OSQP_ERR_DEVICE if a timeout was not reported, OSQP_ERR_ARG for a bad
+ * timeout, OSQP_ERR_CUDA on a CUDA error.  Allocates and frees a few bytes of
+ * device memory; synchronises the device. */
 int32_t osqp_diag_barrier_timeout(double timeout_s);
 
 /* Diagnostic of the sliced sparse layout that osqp_setup builds for every

@@ -130,14 +130,23 @@ __global__ void k_gather(double* __restrict__ dst, const int* __restrict__ idx,
 }
 
 // Barrier diagnostic: CTA `absent` returns without arriving, so the others
-// must time out, record the error and leave.
+// must time out, record the error and leave; at a plain barrier or, with
+// `reduction`, in a reduction.
 __global__ void __launch_bounds__(kThreads) k_barrier_probe(Barrier* bar, int* err, double* part,
                                                              unsigned long long timeout_ns,
-                                                             int absent) {
+                                                             int absent, int reduction,
+                                                             int* passed) {
   __shared__ double sm[kSmemDoubles];
   GridTeam tm{bar, err, part, sm, timeout_ns, 0, 0u};
   if ((int)blockIdx.x == absent) return;
-  tm.sync();
+  bool ok;
+  if (reduction) {
+    const double v[2] = {1.0, 2.0};
+    ok = tm.reduce<2, 2u>(v, [](const double (&)[2]) {});
+  } else {
+    ok = tm.sync();
+  }
+  if (ok && threadIdx.x == 0) atomicAdd(passed, 1);
 }
 
 // Autotuner of a single problem's row partition on the grid team: `reps`
@@ -1167,21 +1176,24 @@ int32_t osqp_diag_barrier_timeout(double timeout_s) {
   }
   Barrier* bar = (Barrier*)mem;
   int* err = (int*)(mem + 256);
+  int* passed = err + 1;  // CTAs that were told of a complete barrier
   double* part = (double*)(mem + 512);
   int rc = OSQP_OK;
-  if (cudaMemset(mem, 0, 512) != cudaSuccess) rc = OSQP_ERR_CUDA;
   unsigned long long tns = (unsigned long long)(timeout_s * 1e9);
   int absent = 1;
-  void* args[] = {&bar, &err, &part, &tns, &absent};
-  if (rc == OSQP_OK &&
-      cudaLaunchCooperativeKernel((const void*)k_barrier_probe, dim3(kBlocks), dim3(kThreads), args,
-                                  0, (cudaStream_t)0) != cudaSuccess)
-    rc = OSQP_ERR_CUDA;
-  if (rc == OSQP_OK && cudaDeviceSynchronize() != cudaSuccess) rc = OSQP_ERR_CUDA;
-  int e = 0;
-  if (rc == OSQP_OK && cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-    rc = OSQP_ERR_CUDA;
-  if (rc == OSQP_OK && e != kDevBarrierTimeout) rc = OSQP_ERR_DEVICE;
+  for (int reduction = 0; rc == OSQP_OK && reduction < 2; ++reduction) {
+    if (cudaMemset(mem, 0, bytes) != cudaSuccess) rc = OSQP_ERR_CUDA;
+    void* args[] = {&bar, &err, &part, &tns, &absent, &reduction, &passed};
+    if (rc == OSQP_OK &&
+        cudaLaunchCooperativeKernel((const void*)k_barrier_probe, dim3(kBlocks), dim3(kThreads),
+                                    args, 0, (cudaStream_t)0) != cudaSuccess)
+      rc = OSQP_ERR_CUDA;
+    if (rc == OSQP_OK && cudaDeviceSynchronize() != cudaSuccess) rc = OSQP_ERR_CUDA;
+    int e[2] = {0, 0};
+    if (rc == OSQP_OK && cudaMemcpy(e, err, sizeof(e), cudaMemcpyDeviceToHost) != cudaSuccess)
+      rc = OSQP_ERR_CUDA;
+    if (rc == OSQP_OK && (e[0] != kDevBarrierTimeout || e[1] != 0)) rc = OSQP_ERR_DEVICE;
+  }
   cudaGetLastError();
   cudaFree(mem);
   return rc;
