@@ -431,9 +431,10 @@ struct GridTeam {
   // cycles of its SM, so those SMs' FP64 pipes set the stage's time (Lasso,
   // 20000 × 200, Ā product: 1300 slices on 81 of 152 SMs).  Used wherever the
   // numbering does not decide which terms share a partial sum.  Measured,
-  // plain -> spread, whole solves in FP64: random QP n = 500 12.4 -> 9.6 ms,
-  // SVM 100 × 10⁴ 30.2 -> 25.3 ms, Lasso 65.2 -> 59.5 ms, portfolio 10⁴ × 100
-  // 357 -> 350 ms.
+  // plain -> spread, whole calls in FP64: random QP n = 500 10.8 -> 9.7 ms,
+  // SVM 100 × 10⁴ 24.0 -> 21.3 ms, Lasso 48.8 -> 43.9 ms, portfolio 10⁴ × 100
+  // 277 -> 269 ms and its matrix update 770 -> 676 us, control step nx = 80
+  // 1432 -> 1347 us.
   __device__ Warps<false> spread() const {
     return {(int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x), nwarps()};
   }
@@ -441,9 +442,9 @@ struct GridTeam {
 
   // Grid barrier with a bounded wait.  The arrival counter only grows
   // during a launch (the host zeroes it before every launch), so barrier
-  // number k is complete once it reaches k·gridDim.x.  Thread 0 arrives with
-  // an acquire-release atomic and spins with acquire loads, so the CTA's
-  // writes before the barrier are visible to every CTA after it.  A CTA that
+  // number k is complete once it reaches k·gridDim.x.  Lane 0 of warp 0
+  // arrives with an acquire-release atomic and spins with acquire loads, so the
+  // CTA's writes before the barrier are visible to every CTA after it.  A CTA that
   // waits longer than timeout_ns records kDevBarrierTimeout and adds
   // kBarrierPoison to the counter, which releases every waiter at once; a
   // counter at or above kBarrierPoison makes every CTA stop at its barrier.
@@ -507,12 +508,12 @@ struct GridTeam {
   // Reduction of at most four slots whose results only one thread turns into
   // scalars: f(results) runs on thread 0 of every CTA, with its writes visible
   // to the CTA on return.  Warp 0 waits for the grid, combines the partials
-  // and runs f in one go, while the other warps wait at a single CTA barrier
-  // (publish_sync, collect and a scalar step after it take four).  The
-  // order of the sums is collect's.  Together with P1's joint fetches,
-  // measured as the gain over the solver without either: random QP n = 500
-  // 1.29× -> 1.39×, Lasso 20000 × 200 1.10× -> 1.25×, SVM 100 × 10⁴ 1.19× ->
-  // 1.37× (FP64).
+  // and runs f in one go, while the other warps wait at two CTA barriers, one
+  // before the arrival and one after f (publish_sync, collect and a scalar
+  // step after it take four).  The order of the sums is collect's.  Measured
+  // against that chain, whole calls: random QP n = 500 9.01 -> 8.89 ms, SVM
+  // 100 × 10⁴ 23.1 -> 22.6 ms, Lasso 20000 × 200 45.3 -> 44.6 ms (FP32-mixed
+  // 35.0 -> 34.5), portfolio 10⁴ × 100 295 -> 293 ms.
   template <int K, unsigned MAXMASK, bool DBL = true, bool MIRROR = false, typename V, class F>
   __device__ bool reduce(const V (&v)[K], F f) {
     static_assert(K <= 4, "four slots at most");
@@ -836,14 +837,14 @@ struct BlockTeam {
   }
 };
 
-// A plain (non-cooperative) launch as a traversal team: no barriers.
-// The one-CTA team of the kernels that also build or stage the problem: their
-// stage R always forms b.  With the second form of the stage the batch kernel
-// was slower in both modes (608 MPC QPs, FP64: 313 -> 362 ms).
+// The one-CTA team of k_batch and k_noalloc: their stage R always forms b.
+// With the second form of the stage the batch kernel was slower in both modes
+// (608 MPC QPs, FP64: 313 -> 362 ms; 314.6 ms as it is).
 struct FullTeam : BlockTeam {
   static constexpr bool kBoundB = false;
 };
 
+// A plain (non-cooperative) launch as a traversal team: no barriers.
 struct PlainTeam {
   static constexpr bool kCtaScope = false;
   __device__ int nthreads() const { return gridDim.x * blockDim.x; }
@@ -1024,10 +1025,10 @@ __device__ __forceinline__ void spmv(const Team& tm, const Sched& S, const int* 
   }
 }
 
-// Sum of a long row's partial value v (chunks r.x … r.x + r.y − 1) after the LAZY product that stored
-// them (a team barrier in between), by one warp: lane k adds chunks k, k+32,
-// … in order, then a fixed xor-shuffle tree, so every lane holds the same
-// total.  All lanes of the warp call it.
+// Sum of a long row's partial value v (chunks r.x … r.x + r.y − 1) after the
+// LAZY product that stored them (a team barrier in between), by one warp: lane
+// k adds chunks k, k+32, … in order, then a fixed xor-shuffle tree, so every
+// lane holds the same total.  All lanes of the warp call it.
 template <typename AT>
 __device__ __forceinline__ AT warp_long_sum(const Sched& S, int2 r, int v) {
   const int lane = threadIdx.x & 31;
@@ -1217,7 +1218,7 @@ __device__ bool scale_stage(Team& tm, const Dev<T>& d, const Params& P, double r
     d.kn_v[k] = T(s);
   });
   foreach_entry(rows, d.as, d.a_ci,
-                        [&](int i, int k) { d.a_v[k] = T(d.E[i] * d.a_raw[k] * d.D[d.a_ci[k]]); });
+                [&](int i, int k) { d.a_v[k] = T(d.E[i] * d.a_raw[k] * d.D[d.a_ci[k]]); });
   for (int j = et; j < n; j += nth) {
     d.q[j] = c * d.D[j] * d.q_raw[j];
     d.Dinv[j] = 1.0 / d.D[j];
@@ -1751,13 +1752,13 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     // same number.  Otherwise the stage runs once more with b, and keeps it for
     // the rest of the solve: residuals mostly fall from check to check, so a
     // floor that binds stays binding (trying again after every check cost a
-    // solve with check_interval = 1 a second R and A0 in each iteration).  Measured in FP64, as the gain over a solver with
-    // none of these stages' forms, before -> after: random QP n = 50 1.06× ->
-    // 1.12× (7.3 -> 6.6 ms in all), MPC step 1.18× -> 1.19×.  FP64 mode only:
-    // in FP32-mixed mode the whole-GPU Lasso gains 1 % and a one-CTA
-    // solve 2 %, but the batch kernel lost a third of its speed at the same
-    // registers and spills, as a second form of the stage (608 MPC QPs 126.8
-    // -> 186.7 ms) and as a predicate in the first (129.3 -> 188.2 ms).
+    // solve with check_interval = 1 a second R and A0 in each iteration).
+    // Measured in FP64, b always formed -> as it is, whole calls: random QP
+    // n = 50 7.76 -> 7.50 ms, SVM 26.8 -> 26.6 ms, random QP n = 500 and Lasso
+    // 0.3 %.  FP64 mode only: in FP32-mixed mode the whole-GPU Lasso gains 1 %
+    // and a one-CTA solve 2 %, but the batch kernel lost a third of its speed
+    // at the same registers and spills, as a second form of the stage (608 MPC
+    // QPs 126.8 -> 186.7 ms) and as a predicate in the first (129.3 -> 188.2 ms).
     if (kBoundB && have_check && !exact_b && colsum < 0.0) {
       double cs[1] = {0.0};
       auto row = [&](int, double* acc) { cs[0] = fmax(cs[0], acc[0]); };
@@ -1775,105 +1776,104 @@ __device__ bool admm_stage(Team& tm, const Dev<T>& d, const Params& P) {
     bool with_b = !kBoundB || !have_check || exact_b;
     bool done;
     for (;;) {
-    {
-      T* __restrict__ r = rbuf(cur);
-      T* __restrict__ u0 = ubuf(cur);
-      auto store = [&](int j, double bj, double acc, double b) {
-        const T rj = T(bj - sigma * xt[j] + acc);
-        r[j] = rj;
-        // here, so that A0 gathers u instead of r and M⁻¹ (with δx and δy
-        // left to the checks, random QP n = 50 FP64: 1.02× -> 1.06×, n = 500
-        // 1.39× -> 1.43×)
-        u0[j] = rj * dinv[j];
-        bv[j] = T(b);
-      };
-      if (!kBoundB || with_b)
-        spmv<2, false, double, T>(
-            rows, d.kn, kn_ci, kn_v,
-            [&](int col, T v, double* acc) {
-              const double vv = (double)v;
-              if (col < n) {
-                acc[0] -= vv * xt[col];
-              } else {
-                acc[0] += vv * um[col - n];
-                acc[1] += vv * wm[col - n];
-              }
-            },
-            [&](int j, double* acc) {
-              const double bj = sigma * x[j] - d.q[j];
-              store(j, bj, acc[0], bj + acc[1]);
-            });
-      else
-        spmv<1, false, double, T>(
-            rows, d.kn, kn_ci, kn_v,
-            [&](int col, T v, double* acc) {
-              const double vv = (double)v;
-              if (col < n) acc[0] -= vv * xt[col];
-              else acc[0] += vv * um[col - n];
-            },
-            [&](int j, double* acc) {
-              const double bj = sigma * x[j] - d.q[j];
-              store(j, bj, acc[0], bj);
-            });
-    }
-    if (!tm.sync()) return false;
+      {
+        T* __restrict__ r = rbuf(cur);
+        T* __restrict__ u0 = ubuf(cur);
+        auto store = [&](int j, double bj, double acc, double b) {
+          const T rj = T(bj - sigma * xt[j] + acc);
+          r[j] = rj;
+          // here, so that A0 gathers u instead of r and M⁻¹ (with δx and δy
+          // left to the checks, random QP n = 50 FP64: 8.3 -> 7.8 ms)
+          u0[j] = rj * dinv[j];
+          bv[j] = T(b);
+        };
+        if (!kBoundB || with_b)
+          spmv<2, false, double, T>(
+              rows, d.kn, kn_ci, kn_v,
+              [&](int col, T v, double* acc) {
+                const double vv = (double)v;
+                if (col < n) {
+                  acc[0] -= vv * xt[col];
+                } else {
+                  acc[0] += vv * um[col - n];
+                  acc[1] += vv * wm[col - n];
+                }
+              },
+              [&](int j, double* acc) {
+                const double bj = sigma * x[j] - d.q[j];
+                store(j, bj, acc[0], bj + acc[1]);
+              });
+        else
+          spmv<1, false, double, T>(
+              rows, d.kn, kn_ci, kn_v,
+              [&](int col, T v, double* acc) {
+                const double vv = (double)v;
+                if (col < n) acc[0] -= vv * xt[col];
+                else acc[0] += vv * um[col - n];
+              },
+              [&](int j, double* acc) {
+                const double bj = sigma * x[j] - d.q[j];
+                store(j, bj, acc[0], bj);
+              });
+      }
+      if (!tm.sync()) return false;
 
-    // PCG on K = P̄ + σI + ĀᵀRĀ in the single-reduction form of Chronopoulos
-    // and Gear: per iteration one stage that updates p, s = Kp, x̃, r, u = M⁻¹r
-    // and computes t = RĀu with u formed on the fly, and one stage that forms
-    // w = Ku and the two inner products (r,u), (w,u).  r, s, w and t are
-    // double-buffered so that gathers never see a vector being rewritten.
-    // --- A0: t = RĀu with the u = M⁻¹r that R left; (r,u), ‖r‖∞, ‖b‖∞ (or half
-    // its bound)
-    T red3t[3];
-    {
-      const T* __restrict__ r = rbuf(cur);
-      const T* __restrict__ u = ubuf(cur);
-      T* __restrict__ t = ubuf(cur) + n;
-      T a0 = T(0), a1 = T(0), a2 = T(0);
-      for (int j = tid; j < n; j += nth) {
-        const T rj = r[j];
-        a0 += rj * u[j];
-        a1 = fmax(a1, fabs(rj));
-        a2 = fmax(a2, fabs(bv[j]));
+      // PCG on K = P̄ + σI + ĀᵀRĀ in the single-reduction form of Chronopoulos
+      // and Gear: per iteration one stage that updates p, s = Kp, x̃, r,
+      // u = M⁻¹r and computes t = RĀu, and one stage that forms w = Ku and the
+      // two inner products (r,u), (w,u).  r, s, w and t are double-buffered so
+      // that gathers never see a vector being rewritten.
+      // --- A0: t = RĀu with the u = M⁻¹r that R left; (r,u), ‖r‖∞, ‖b‖∞ (or half
+      // its bound)
+      T red3t[3];
+      {
+        const T* __restrict__ r = rbuf(cur);
+        const T* __restrict__ u = ubuf(cur);
+        T* __restrict__ t = ubuf(cur) + n;
+        T a0 = T(0), a1 = T(0), a2 = T(0);
+        for (int j = tid; j < n; j += nth) {
+          const T rj = r[j];
+          a0 += rj * u[j];
+          a1 = fmax(a1, fabs(rj));
+          a2 = fmax(a2, fabs(bv[j]));
+        }
+        if (kBoundB && !with_b) {
+          double w = 0.0;
+          for (int i = et; i < m; i += nth) w = fmax(w, fabs(wm[i]));
+          a2 = fmax(a2, T(colsum * w));
+        }
+        red3t[0] = a0;
+        red3t[1] = a1;
+        red3t[2] = a2;
+        spmv<1, false, T, T>(
+            prows, d.as, a_ci, a_v,
+            [&](int col, T v, T* acc) { acc[0] += v * u[col]; },
+            [&](int i, T* acc) { t[i] = rhoT[i] * acc[0]; });
       }
-      if (kBoundB && !with_b) {
-        double w = 0.0;
-        for (int i = et; i < m; i += nth) w = fmax(w, fabs(wm[i]));
-        a2 = fmax(a2, T(colsum * w));
-      }
-      red3t[0] = a0;
-      red3t[1] = a1;
-      red3t[2] = a2;
-      spmv<1, false, T, T>(
-          prows, d.as, a_ci, a_v,
-          [&](int col, T v, T* acc) { acc[0] += v * u[col]; },
-          [&](int i, T* acc) { t[i] = rhoT[i] * acc[0]; });
-    }
-    if (!tm.template reduce<3, 6u, true, kF32>(red3t, [&](const double (&red3)[3]) {
-          // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
-          double tol;
-          int flag = 0;
-          if (!kBoundB || with_b) {
-            const double bnorm = red3[2];
-            tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
-                       have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
-                                  : 0.1 * P.pcg_kappa * bnorm);
-          } else {
-            // both terms of the bound are at most red3[2] (rounded to T)
-            tol = fmax(P.pcg_reduce * red3[1], P.pcg_kappa * fmin(rp_bar, rd_bar));
-            if (!(P.pcg_floor * (2.02 * red3[2]) <= tol)) flag = 2;
-          }
-          scal[0] = red3[0];  // γ = (r, M⁻¹r)
-          scal[3] = tol;
-          if (kF32) *ftol = (float)tol;
-          *sflag = flag ? flag : !(red3[1] > tol);
-        }))
-      return false;
-    const int flag = *sflag;
-    done = flag != 0;
-    if (!kBoundB || flag != 2) break;
-    exact_b = with_b = true;
+      if (!tm.template reduce<3, 6u, true, kF32>(red3t, [&](const double (&red3)[3]) {
+            // PCG accuracy (reading of "up to some predefined accuracy", §3.1).
+            double tol;
+            int flag = 0;
+            if (!kBoundB || with_b) {
+              const double bnorm = red3[2];
+              tol = fmax(fmax(P.pcg_floor * bnorm, P.pcg_reduce * red3[1]),
+                         have_check ? P.pcg_kappa * fmin(rp_bar, rd_bar)
+                                    : 0.1 * P.pcg_kappa * bnorm);
+            } else {
+              // both terms of the bound are at most red3[2] (rounded to T)
+              tol = fmax(P.pcg_reduce * red3[1], P.pcg_kappa * fmin(rp_bar, rd_bar));
+              if (!(P.pcg_floor * (2.02 * red3[2]) <= tol)) flag = 2;
+            }
+            scal[0] = red3[0];  // γ = (r, M⁻¹r)
+            scal[3] = tol;
+            if (kF32) *ftol = (float)tol;
+            *sflag = flag ? flag : !(red3[1] > tol);
+          }))
+        return false;
+      const int flag = *sflag;
+      done = flag != 0;
+      if (!kBoundB || flag != 2) break;
+      exact_b = with_b = true;
     }
     if constexpr (kF32) {
       cg_g = ff{fmir[0], fmir[1]};
