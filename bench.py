@@ -60,14 +60,14 @@ WORKLOADS = {
 }
 PARAM_LEN = {"lasso_path": 100, "mpc_loop": 100, "portfolio_bt": 960}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# the dominant kernel, from one ncu capture of the same command with the
-# kernels as they are now; for the batch, the capture of the first 608
+# the dominant kernel, from one single-pass ncu capture of the same command
+# with the kernels as they are now; for the batch, the capture of the first 608
 # problems scaled by the problems of the launch.  Absent: not captured
 # since the kernels last changed.  The single-problem figure holds for the
 # row partitions it was captured with (group widths of Kn and Ā).
-TRAFFIC = {("lasso", "fp64"): 20.403456e6}
+TRAFFIC = {("lasso", "fp64"): 21.120000e6}
 TRAFFIC_GROUPS = {("lasso", "fp64"): (2, 2)}
-TRAFFIC_BATCH_PER_PROBLEM = {"fp32": 3.380327168e9 / 608}
+TRAFFIC_BATCH_PER_PROBLEM = {"fp32": 3.025579776e9 / 608}
 # Mean time per QP and mean iterations per QP that the paper reports for the
 # same sequences (OSQP direct method on a CPU; context only)
 PARAM_PAPER = {
